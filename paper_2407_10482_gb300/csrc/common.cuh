@@ -414,10 +414,9 @@ __device__ __forceinline__ void load_entry<NGPRT_BF16>(const void* base, uint32_
     const uint32_t w[4] = {q.x, q.y, q.z, q.w};
 #pragma unroll
     for (int k = 0; k < 4; ++k) {
-        __nv_bfloat162 h = *reinterpret_cast<const __nv_bfloat162*>(&w[k]);
-        float2 f = __bfloat1622float2(h);
-        v[2 * k] = f.x;
-        v[2 * k + 1] = f.y;
+        // a BF16 value is the upper half of its FP32 word
+        v[2 * k] = __uint_as_float(w[k] << 16);
+        v[2 * k + 1] = __uint_as_float(w[k] & 0xFFFF0000u);
     }
 }
 
@@ -458,7 +457,7 @@ __device__ __forceinline__ void load_channels(const void* base, uint32_t vertex,
         for (int k = 0; k < NC / 2; ++k) {
             float2 f;
             if constexpr (DT == NGPRT_F16) f = __half22float2(*reinterpret_cast<const __half2*>(&w[k]));
-            else f = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&w[k]));
+            else f = make_float2(__uint_as_float(w[k] << 16), __uint_as_float(w[k] & 0xFFFF0000u));
             v[2 * k] = f.x;
             v[2 * k + 1] = f.y;
         }

@@ -56,13 +56,14 @@ struct MarchParams {
 // Ray of this thread (false if the lane has none): origin and unnormalised
 // double-float direction.
 // tile_of_warp: the warp's camera tile (mode 0) or run of 32 rays (modes 1, 2), or
-// -1 for the one of its own index.
+// -1 for the one of its own index; lane_of_tile: the ray within it, or -1 for the
+// thread's lane.
 __device__ __forceinline__ bool thread_ray(const MarchParams& p, int64_t& ray, float o[3], df d[3],
-                                           int64_t tile_of_warp = -1) {
+                                           int64_t tile_of_warp = -1, int lane_of_tile = -1) {
+    const int lane = lane_of_tile >= 0 ? lane_of_tile : (int)(threadIdx.x & 31);
     if (p.mode == 0) {
         const int64_t warp =
             tile_of_warp >= 0 ? tile_of_warp : (((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5);
-        const int lane = threadIdx.x & 31;
         const int64_t view = warp / p.tiles_per_view;
         if (view >= p.n_cams) return false;
         const int tile = (int)(warp - view * p.tiles_per_view);
@@ -73,7 +74,7 @@ __device__ __forceinline__ bool thread_ray(const MarchParams& p, int64_t& ray, f
         camera_ray_df(p.cams.c[view], col, row, o, d);
         return true;
     }
-    ray = tile_of_warp >= 0 ? tile_of_warp * 32 + (threadIdx.x & 31) : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    ray = tile_of_warp >= 0 ? tile_of_warp * 32 + lane : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (ray >= p.n_rays) return false;
     if (p.mode == 1) {
         int64_t id = p.pixel_ids[ray];
@@ -157,6 +158,82 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
 constexpr int kLevelUnroll = NGPRT_LEVEL_UNROLL;
 constexpr int kScatterUnroll = NGPRT_SCATTER_UNROLL;
 
+// Where the gates of Eq. 8 come from.  FP32 and BF16 tables: each level interpolates its
+// own two logits when its turn comes (8 loads of one pair).  The 2L sums are then not
+// all held at once, nothing passes through shared memory (which is carved out of L1),
+// and the level loop has the registers that the 40 coarse channels took: hd 1080p FP32
+// 12.52 -> 11.52 ms with the blocks below, BF16 (1283 x 721) 7.2 -> 5.0 ms (it spilled
+// 460 B a thread).  FP16 tables keep the coarse rows in one pass with the gates in
+// shared memory: half2 sums need half the registers, and the extra loads cost more
+// than they free (6.77 ms against 7.51).
+template <int DT, int AGG>
+constexpr bool fly_gates() {
+    return AGG == NGPRT_AGG_SEPARATE_V && DT != NGPRT_F16;
+}
+
+// The first NF of a coarse row's NC channels, FP32 or BF16 (NF = 8: the loads that the
+// whole row's alignment allows).
+template <int DT, int NC, int NF>
+__device__ __forceinline__ void load_row_channels(const void* base, uint32_t vertex, float v[NF]) {
+    if constexpr (NF == NC) load_channels<DT, NC>(base, vertex, v);
+    else if constexpr (DT == NGPRT_F32) {
+        static_assert(NF == kNFeat, "the feature channels");
+        const float* p = static_cast<const float*>(base) + (size_t)vertex * NC;
+        if constexpr (NC % 8 == 0) load_entry<NGPRT_F32>(p, 0, v);
+        else if constexpr (NC % 4 == 0) {
+#pragma unroll
+            for (int k = 0; k < NF / 4; ++k) {
+                const float4 q = __ldg(reinterpret_cast<const float4*>(p) + k);
+                v[4 * k] = q.x; v[4 * k + 1] = q.y; v[4 * k + 2] = q.z; v[4 * k + 3] = q.w;
+            }
+        } else {
+#pragma unroll
+            for (int k = 0; k < NF / 2; ++k) {
+                const float2 q = __ldg(reinterpret_cast<const float2*>(p) + k);
+                v[2 * k] = q.x; v[2 * k + 1] = q.y;
+            }
+        }
+    } else {
+        static_assert(NF == kNFeat, "the feature channels");
+        const uint16_t* p = static_cast<const uint16_t*>(base) + (size_t)vertex * NC;
+        if constexpr (NC % 8 == 0) load_entry<NGPRT_BF16>(p, 0, v);
+        else {
+#pragma unroll
+            for (int k = 0; k < NF / 2; ++k) {
+                const uint32_t q = __ldg(reinterpret_cast<const uint32_t*>(p) + k);
+                v[2 * k] = __uint_as_float(q << 16);
+                v[2 * k + 1] = __uint_as_float(q & 0xFFFF0000u);
+            }
+        }
+    }
+}
+
+// Gates omega^l, beta^l of one level from its two logits at the 8 coarse corners.
+template <int DT, int NC>
+__device__ __forceinline__ void level_gates(const Grid& g, uint32_t cb, uint32_t sy, uint32_t sz, const float w[3],
+                                            int l, int attn_mode, float& om, float& be) {
+    if (attn_mode == 1) {
+        om = be = 1.0f;
+        return;
+    }
+    float2 lg = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const uint32_t v = cb + (uint32_t)(c & 1) + sy * (uint32_t)((c >> 1) & 1) + sz * (uint32_t)((c >> 2) & 1);
+        const float cw = corner_w(w, c);
+        float2 q;
+        if constexpr (DT == NGPRT_F32) {
+            q = __ldg(reinterpret_cast<const float2*>(static_cast<const float*>(g.coarse) + (size_t)v * NC + kNFeat) + l);
+        } else {
+            const uint32_t x = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(g.coarse) + (size_t)v * NC + kNFeat) + l);
+            q = make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
+        }
+        lg = ffma2(make_float2(cw, cw), q, lg);
+    }
+    om = gate_sigmoid(lg.x);
+    be = attn_mode == 2 ? om : gate_sigmoid(lg.y);
+}
+
 // Eq. 6-8 at unit-cube position u: f = f~ + Att(f^1..f^L; a), or one of the
 // aggregations of Table 3 (AGG, an ngprt_aggregation).  The coarse fetch
 // interpolates the coarse grid's channels (f~ and, for the spatially variant forms,
@@ -181,6 +258,8 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
     // level) and each level's gated sum is taken in mixed precision (FP16 factors,
     // FP32 sum), without converting the level's features
     constexpr bool kHalfGates = DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V && !kKeep;
+    constexpr bool kFly = fly_gates<DT, AGG>() && !kKeep;
+    constexpr int NF = kFly ? kNFeat : NC;  // channels taken from the coarse rows up front
     uint32_t ufx[3] = {0u, 0u, 0u};
     if constexpr (DT != NGPRT_F32) {
 #pragma unroll
@@ -190,7 +269,7 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
     float w[3];
 #pragma unroll
     for (int a = 0; a < 3; ++a) table_cell<DT>(u[a], ufx[a], g.R_C, b[a], w[a]);
-    float2 acc[NC / 2];
+    float2 acc[NF / 2];
     uint32_t cb, sy, sz;
     coarse_base(g, b, cb, sy, sz);
     if constexpr (DT == NGPRT_F16) {
@@ -222,16 +301,16 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
         }
     } else {
 #pragma unroll
-        for (int ch = 0; ch < NC / 2; ++ch) acc[ch] = make_float2(0.0f, 0.0f);
+        for (int ch = 0; ch < NF / 2; ++ch) acc[ch] = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const uint32_t v = cb + (uint32_t)(c & 1) + sy * (uint32_t)((c >> 1) & 1) + sz * (uint32_t)((c >> 2) & 1);
-            float val[NC];
-            load_channels<DT, NC>(g.coarse, v, val);
+            float val[NF];
+            load_row_channels<DT, NC, NF>(g.coarse, v, val);
             const float cw = corner_w(w, c);
             const float2 cw2 = make_float2(cw, cw);
 #pragma unroll
-            for (int ch = 0; ch < NC / 2; ++ch) acc[ch] = ffma2(cw2, make_float2(val[2 * ch], val[2 * ch + 1]), acc[ch]);
+            for (int ch = 0; ch < NF / 2; ++ch) acc[ch] = ffma2(cw2, make_float2(val[2 * ch], val[2 * ch + 1]), acc[ch]);
         }
     }
 #pragma unroll
@@ -239,7 +318,7 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
         f[2 * ch] = acc[ch].x;
         f[2 * ch + 1] = acc[ch].y;
     }
-    if constexpr (kGated && !kHalfGates) {
+    if constexpr (kGated && !kHalfGates && !kFly) {
 #pragma unroll
         for (int l = 0; l < L; ++l) {
             float om, be;
@@ -382,7 +461,12 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
             }
         } else if constexpr (!kHalfGates) {
             // packed pairs: each half is the scalar fmaf, bit for bit
-            const float om = gates[(2 * l) * stride], be = gates[(2 * l + 1) * stride];
+            float om, be;
+            if constexpr (kFly) level_gates<DT, NC>(g, cb, sy, sz, w, l, attn_mode, om, be);
+            else {
+                om = gates[(2 * l) * stride];
+                be = gates[(2 * l + 1) * stride];
+            }
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
                 const float2 r = ffma2(make_float2(ch == 0 ? om : be, be), fl[ch], make_float2(f[2 * ch], f[2 * ch + 1]));
@@ -422,6 +506,15 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
             f[k] += o;
         }
     }
+}
+
+// Shared-memory floats per thread that sample_features parks its gates in (forward
+// form).  What shared memory takes is lost to L1, which holds the coarse rows and the
+// dense levels.
+template <int L, int DT, int AGG>
+__host__ __device__ constexpr int gate_floats() {
+    if (AGG == NGPRT_AGG_SUM || AGG == NGPRT_AGG_MLP || fly_gates<DT, AGG>()) return 0;
+    return DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V ? L : 2 * L;
 }
 
 // World length of a step whose contracted image stays within rho of its start (so
@@ -693,10 +786,10 @@ struct ForwardSampler {
 // Ray set-up shared by every pass: this thread's ray and its domain interval
 // (false if the lane has no ray; hit = the interval is not empty).
 __device__ __forceinline__ bool ray_setup(const MarchParams& p, int64_t& ray, Ray& ry, bool& hit,
-                                          int64_t tile_of_warp = -1) {
+                                          int64_t tile_of_warp = -1, int lane_of_tile = -1) {
     float o[3];
     df d[3];
-    if (!thread_ray(p, ray, o, d, tile_of_warp)) return false;
+    if (!thread_ray(p, ray, o, d, tile_of_warp, lane_of_tile)) return false;
     float t_lo = -INFINITY, t_hi = INFINITY;
     if (p.t_interval && !p.fb_a_hat) {
         t_lo = p.t_interval[2 * ray];
@@ -714,18 +807,19 @@ __device__ __forceinline__ bool ray_setup(const MarchParams& p, int64_t& ray, Ra
 // 32 listed rays) from the counter until none are left: a warp that finishes early
 // starts another tile instead of idling until its block's slowest warp ends (fitted
 // hd scene, 1080p: FP16 9.46 -> 8.98 ms, FP32 16.05 -> 15.60 ms).
-// Blocks per SM the register allocation must allow (measured at 1080p on the
-// fitted hd scene, L = 16, and earlier on the paper shape, L = 4): FP32 tables with
-// 4 or more levels are fastest at 5 (102 registers; 16.1 ms against 16.2 at 6 and
-// 18.0 at 8), FP16 tables at 8 (64 registers; 9.5 ms against 9.6 at 7 and 9.9 at
-// 6), BF16 tables (interpolated in FP32) at 7; FP32 with fewer levels keeps 8.  The
-// MLP aggregation keeps its 64 hidden units in registers.
+// Blocks per SM the register allocation must allow (hd scene, L = 16): FP32 tables with 4
+// or more levels 7 (72 registers; 1080p 11.5 ms against 12.0 at 5, 11.7 at 6 and 12.0 at
+// 8), FP16 tables 8 (64 registers; 6.77 ms against 6.83 at 7), BF16 tables 8 (5.00 ms
+// against 5.12 at 7 and 5.23 at 10); FP32 with fewer levels 8.  The other aggregation
+// forms of FP32 and BF16 tables hold more and keep 5 and 7; the MLP form keeps its 64
+// hidden units in registers.
 template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V>
 constexpr int march_min_blocks() {
     if (AGG == NGPRT_AGG_MLP) return 3;
     if (NGPRT_MARCH_MIN_BLOCKS > 0) return NGPRT_MARCH_MIN_BLOCKS;
-    if (DT == NGPRT_F32) return L >= 4 ? 5 : 8;
-    return DT == NGPRT_F16 ? 8 : 7;
+    if (DT == NGPRT_F16) return 8;
+    if (AGG != NGPRT_AGG_SEPARATE_V) return DT == NGPRT_BF16 ? 7 : L >= 4 ? 5 : 8;
+    return DT == NGPRT_F32 && L >= 4 ? 7 : 8;
 }
 
 template <int L, int DT, int AGG>
@@ -790,7 +884,7 @@ int resident_blocks(Kernel k, size_t shm) {
 
 template <int L, int DT, int AGG>
 void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
-    const size_t shm = (size_t)2 * L * 128 * sizeof(float);  // attention gates of the block's rays
+    const size_t shm = (size_t)gate_floats<L, DT, AGG>() * 128 * sizeof(float);  // attention gates of the block's rays
     if (p.tile_counter) {
         // this instantiation's resident blocks, per device, found once
         static int cache[16] = {0};
