@@ -266,6 +266,24 @@ int32_t ngprt_occupancy_visibility(const ngprt_scene* scene, const ngprt_occ* oc
                                    int32_t R, uint8_t* vis, void* stream);
 
 /*
+ * The passes that read the density path alone (ngprt_occupancy_from_density,
+ * ngprt_occupancy_visibility, ngprt_distortion_loss) in forms with a workspace: with
+ * ngprt_density_scratch_bytes(scene, n_rays) bytes (n_rays = 0 for
+ * ngprt_occupancy_from_density_ws; 0 bytes where the scene has no faster form) they copy
+ * the tables' density channel there first and, for camera pixel lists, take the rays in
+ * pixel-tile order.  The results are those of the forms without; a NULL or smaller
+ * workspace gives exactly those forms.
+ */
+size_t ngprt_density_scratch_bytes(const ngprt_scene* scene, int64_t n_rays);
+int32_t ngprt_occupancy_from_density_ws(const ngprt_scene* scene, const ngprt_render_opts* opts, int32_t R,
+                                        float sigma_thr, uint8_t* occ_out, float* sigma_out, void* workspace,
+                                        size_t ws_bytes, void* stream);
+int32_t ngprt_occupancy_visibility_ws(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
+                                      int32_t n_cams, const int32_t* pixel_ids, const float* rays_o,
+                                      const float* rays_d, int64_t n_rays, const ngprt_render_opts* opts, float w_thr,
+                                      int32_t R, uint8_t* vis, void* workspace, size_t ws_bytes, void* stream);
+
+/*
  * ngprt_dilate: out[v] = max of occ over the voxels within `radius` of v along
  *   every axis (a (2 radius + 1)^3 box clipped by the grid's faces), then 0 wherever
  *   mask[v] == 0 (mask NULL: no mask; e.g. the density occupancy, so that the render
@@ -344,6 +362,12 @@ int32_t ngprt_shade(const ngprt_scene* scene, const float* ray_state, int64_t n_
  */
 size_t ngprt_render_backward_workspace_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
                                              int64_t n_rays);
+/* Bytes with which ngprt_render_backward is fastest (>= the workspace bytes; about 11 KB
+ * a ray at L = 16, for at most 2^18 rays at a time): it then records the samples and sums
+ * each ray's records per grid cell before adding to the gradients.  Any workspace from
+ * ngprt_render_backward_workspace_bytes on is accepted; a smaller one than this takes
+ * the form that adds every sample by itself. */
+size_t ngprt_render_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts, int64_t n_rays);
 int32_t ngprt_render_backward(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
                               int32_t n_cams, const int32_t* pixel_ids, const float* rays_o,
                               const float* rays_d, int64_t n_rays, const ngprt_render_opts* opts,
@@ -441,10 +465,20 @@ int32_t ngprt_huber_loss(const float* rgb, const float* target, int64_t n, float
  */
 size_t ngprt_distortion_backward_workspace_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
                                                  int64_t n_rays);
+/* Bytes with which ngprt_distortion_backward is fastest, as
+ * ngprt_render_backward_scratch_bytes (any smaller workspace the call accepts without
+ * them is still accepted). */
+size_t ngprt_distortion_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
+                                               int64_t n_rays);
 int32_t ngprt_distortion_loss(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
                               int32_t n_cams, const int32_t* pixel_ids, const float* rays_o, const float* rays_d,
                               int64_t n_rays, const ngprt_render_opts* opts, float scale, float* dist_state,
                               float* loss, void* stream);
+/* ngprt_distortion_loss with a workspace (see ngprt_density_scratch_bytes). */
+int32_t ngprt_distortion_loss_ws(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
+                                 int32_t n_cams, const int32_t* pixel_ids, const float* rays_o, const float* rays_d,
+                                 int64_t n_rays, const ngprt_render_opts* opts, float scale, float* dist_state,
+                                 float* loss, void* workspace, size_t ws_bytes, void* stream);
 int32_t ngprt_distortion_backward(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
                                   int32_t n_cams, const int32_t* pixel_ids, const float* rays_o, const float* rays_d,
                                   int64_t n_rays, const ngprt_render_opts* opts, const float* dist_state, float scale,

@@ -8,7 +8,7 @@
 // Kernel 2 (march_backward_kernel, backward_march.cuh): per ray, the march again
 // and the reverse of compositing, gates and trilinear gathers, added atomically to
 // the table, coarse-grid and invariant-logit gradients.
-#include "backward_march.cuh"
+#include "records.cuh"
 
 namespace ngprt {
 namespace {
@@ -258,7 +258,123 @@ void launch_shade_bwd(const ShadeBwdParams& s, cudaStream_t st) {
     shade_backward_kernel<WIDTH, LAYERS><<<blocks, 128, smem, st>>>(s);
 }
 
+__global__ void bin_count_kernel(const __grid_constant__ BinParams p) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < p.n) atomicAdd(p.bins + bin_of(p, i), 1u);
+}
+
+// Exclusive prefix of the bins, in place: one block, each thread a run of n / 1024.
+__global__ void __launch_bounds__(1024) bin_scan_kernel(uint32_t* bins, int n) {
+    __shared__ uint32_t part[32];
+    const int per = (n + 1023) / 1024, lo = min(n, (int)threadIdx.x * per), hi = min(n, lo + per);
+    uint32_t sum = 0;
+    for (int k = lo; k < hi; ++k) sum += bins[k];
+    uint32_t x = sum;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    if (lane == 31) part[warp] = x;
+    __syncthreads();
+    if (warp == 0) {
+        uint32_t v = part[lane];
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+            const uint32_t y = __shfl_up_sync(0xffffffffu, v, o);
+            if (lane >= o) v += y;
+        }
+        part[lane] = v;
+    }
+    __syncthreads();
+    uint32_t at = x - sum + (warp ? part[warp - 1] : 0u);
+    for (int k = lo; k < hi; ++k) {
+        const uint32_t c = bins[k];
+        bins[k] = at;
+        at += c;
+    }
+}
+
+__global__ void bin_place_kernel(const __grid_constant__ BinParams p) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < p.n) p.perm[atomicAdd(p.bins + bin_of(p, i), 1u)] = (int32_t)i;
+}
+
 }  // namespace
+
+// Channel 0 of every table row.  Four rows a thread: 1 float of each 32-byte sector in,
+// 16 bytes out.
+static __global__ void plane_kernel(const float* __restrict__ tables, int64_t n, float* __restrict__ plane) {
+    const int64_t i = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) * 4;
+    if (i + 4 <= n) {
+        float4 v;
+        v.x = __ldg(tables + 8 * i);
+        v.y = __ldg(tables + 8 * i + 8);
+        v.z = __ldg(tables + 8 * i + 16);
+        v.w = __ldg(tables + 8 * i + 24);
+        *reinterpret_cast<float4*>(plane + i) = v;
+    } else {
+        for (int64_t k = i; k < n; ++k) plane[k] = __ldg(tables + 8 * k);
+    }
+}
+
+void density_scratch(MarchParams& p, int64_t entries, bool order, void* scratch, cudaStream_t st) {
+    const PlaneLayout a = plane_layout(entries, order ? p.n_rays : 0);
+    char* base = reinterpret_cast<char*>(((uintptr_t)scratch + 255) & ~(uintptr_t)255);
+    float* plane = reinterpret_cast<float*>(base + a.plane);
+    plane_kernel<<<(unsigned)((entries + 1023) / 1024), 256, 0, st>>>(static_cast<const float*>(p.g.tables), entries, plane);
+    p.plane = plane;
+    p.perm = nullptr;
+    if (order && p.n_rays >= kRecordMinRays && p.n_rays <= 0x7FFFFFFF)
+        p.perm = bin_rays(p, reinterpret_cast<uint32_t*>(base + a.bins), reinterpret_cast<int32_t*>(base + a.perm), st);
+}
+
+const int32_t* bin_rays(const MarchParams& m, uint32_t* bins, int32_t* perm, cudaStream_t st) {
+    if (m.mode != 1) return nullptr;
+    BinParams b;
+    b.pixel_ids = m.pixel_ids;
+    b.n = m.n_rays;
+    b.n_cams = m.n_cams;
+    b.W = m.W;
+    b.H = m.H;
+    b.bins = bins;
+    b.perm = perm;
+    int64_t n_bins = 0;
+    for (b.tile = 32;; b.tile *= 2) {
+        b.tx = (m.W + b.tile - 1) / b.tile;
+        b.ty = (m.H + b.tile - 1) / b.tile;
+        n_bins = (int64_t)b.tx * b.ty * m.n_cams;
+        if (n_bins <= kMaxBins) break;
+    }
+    const unsigned blocks = (unsigned)((b.n + 255) / 256);
+    cudaMemsetAsync(bins, 0, (size_t)n_bins * sizeof(uint32_t), st);
+    bin_count_kernel<<<blocks, 256, 0, st>>>(b);
+    bin_scan_kernel<<<1, 1024, 0, st>>>(bins, (int)n_bins);
+    bin_place_kernel<<<blocks, 256, 0, st>>>(b);
+    return perm;
+}
+
+// Eq. 8's reverse march: by records where the scratch is there, else in one kernel.
+template <int L>
+static void launch_bwd_l(const MarchBwdParams& p, dim3 grid, void* scratch, cudaStream_t st) {
+    if (!scratch) {
+        launch_bwd<L, NGPRT_AGG_SEPARATE_V>(p, grid, st);
+        return;
+    }
+    RecParams r;
+    memset(&r, 0, sizeof r);
+    r.m = p.m;
+    r.cot = p.cot;
+    r.g_tables = p.g_tables;
+    r.g_coarse = p.g_coarse;
+    launch_records<L, false>(r, scratch, st, [&](const RecParams& q, unsigned blocks) {
+        MarchBwdParams rest = p;
+        rest.list = q.list;
+        rest.n_list = q.n_list;
+        launch_bwd<L, NGPRT_AGG_SEPARATE_V>(rest, dim3(blocks), st);
+    });
+}
 
 int32_t make_grid(const ngprt_scene* s, Grid& g, const char* fn);
 int32_t make_occ(const ngprt_occ* o, OccView& v, const char* fn);
@@ -287,6 +403,13 @@ extern "C" size_t ngprt_render_backward_workspace_bytes(const ngprt_scene* scene
         b += 256 + (size_t)n_rays * (size_t)ms * (size_t)(kNFeat * (scene->L + 1)) * sizeof(float);
     }
     return b;
+}
+
+extern "C" size_t ngprt_render_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
+                                                      int64_t n_rays) {
+    const size_t b = ngprt_render_backward_workspace_bytes(scene, opts, n_rays);
+    if (!b || scene->aggregation != NGPRT_AGG_SEPARATE_V) return b;
+    return b + record_scratch_bytes(scene->L, false, n_rays);
 }
 
 extern "C" int32_t ngprt_render_backward(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
@@ -386,13 +509,16 @@ extern "C" int32_t ngprt_render_backward(const ngprt_scene* scene, const ngprt_o
             launch_bwd_agg_mlp_wgrad(scene->L, p, scene->agg_mlp, g_agg_mlp, st);
         return cuda_status(fn);
     }
+    void* scratch = nullptr;
+    const size_t rec = record_scratch_bytes(scene->L, false, n_rays);
+    if (rec && ws_bytes >= cot_bytes(n_rays) + rec) scratch = static_cast<char*>(workspace) + cot_bytes(n_rays);
     switch (scene->L) {
-        case 1: launch_bwd<1, NGPRT_AGG_SEPARATE_V>(p, grid, st); break;
-        case 2: launch_bwd<2, NGPRT_AGG_SEPARATE_V>(p, grid, st); break;
-        case 3: launch_bwd<3, NGPRT_AGG_SEPARATE_V>(p, grid, st); break;
-        case 4: launch_bwd<4, NGPRT_AGG_SEPARATE_V>(p, grid, st); break;
-        case 8: launch_bwd<8, NGPRT_AGG_SEPARATE_V>(p, grid, st); break;
-        default: launch_bwd<16, NGPRT_AGG_SEPARATE_V>(p, grid, st); break;
+        case 1: launch_bwd_l<1>(p, grid, scratch, st); break;
+        case 2: launch_bwd_l<2>(p, grid, scratch, st); break;
+        case 3: launch_bwd_l<3>(p, grid, scratch, st); break;
+        case 4: launch_bwd_l<4>(p, grid, scratch, st); break;
+        case 8: launch_bwd_l<8>(p, grid, scratch, st); break;
+        default: launch_bwd_l<16>(p, grid, scratch, st); break;
     }
     return cuda_status(fn);
 }

@@ -27,7 +27,17 @@ struct MarchBwdParams {
     int64_t rec_capacity;
     const float* dist_state;  // distortion mode: per ray (L_dist, W, S, 0) of the forward
     float dist_scale;         // distortion mode: dL_total / dL_dist
+    const int2* list;         // only these rays, from these samples on (NULL: all rays, whole)
+    const int32_t* n_list;    // their count (device)
 };
+
+// The ray `ray` of the batch set up for its march; false when its interval is empty.
+__device__ __forceinline__ bool ray_setup_at(const MarchParams& p, int64_t ray, Ray& ry) {
+    float o[3];
+    df d[3];
+    ray_of(p, ray, o, d);
+    return ray_interval(p.g.bounded, o, d, p.opts.t_min, p.opts.r_far, -INFINITY, INFINITY, ry);
+}
 
 // Floats of one MLP-form sample record: the level features x (8L) and the feature
 // cotangent g_f (8).
@@ -252,6 +262,7 @@ struct BackwardSampler {
     int64_t rec_capacity;
     float dW = 0.0f, dS = 0.0f, dG = 0.0f;                         // distortion running sums
     float dW_tot = 0.0f, dS_tot = 0.0f, dG_tot = 0.0f, d_scale = 0.0f;  // and the ray's totals
+    int skip = 0;             // samples whose gradients are elsewhere already
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
         float f[8];
         const float gq[7] = {gCd[0], gCd[1], gCd[2], gF[0], gF[1], gF[2], gF[3]};
@@ -280,6 +291,11 @@ struct BackwardSampler {
             S_le = fmaf(w, qg, S_le);
             const float g_sigma = delta * (T_next * qg - (S_tot - S_le));
             gs = g_sigma * expf(fminf(f[0], 15.0f));
+        }
+        if (skip > 0) {
+            --skip;
+            T = T_next;
+            return T < t_term;
         }
         scatter_features<L, AGG, kDist>(g, u, attn_mode, gs, w, gq, gates, blockDim.x, g_tables, g_coarse);
         if constexpr (AGG == NGPRT_AGG_MLP) {
@@ -322,8 +338,19 @@ __global__ void __launch_bounds__(128, NGPRT_BWD_MIN_BLOCKS) march_backward_kern
     }
     int64_t ray;
     Ray ry;
-    bool hit = false;
-    const bool live = ray_setup(p.m, ray, ry, hit) && hit;
+    bool hit = false, live;
+    int skip = 0;
+    if (p.list) {
+        const int at = blockIdx.x * blockDim.x + threadIdx.x;
+        live = at < *p.n_list;
+        if (live) {
+            ray = p.list[at].x;
+            skip = p.list[at].y;
+            live = ray_setup_at(p.m, ray, ry);
+        }
+    } else {
+        live = ray_setup(p.m, ray, ry, hit) && hit;
+    }
     if constexpr (NI == 0) {
         if (!live) return;
     }
@@ -335,7 +362,7 @@ __global__ void __launch_bounds__(128, NGPRT_BWD_MIN_BLOCKS) march_backward_kern
                                               {0.0f, 0.0f, 0.0f}, {0.0f, 0.0f, 0.0f, 0.0f}, 0.0f, 0.0f,
                                               p.g_tables, p.g_coarse, slots, p.records, p.n_records,
                                               p.rec_capacity, 0.0f, 0.0f, 0.0f, ds.y, ds.z, 2.0f * ds.x,
-                                              p.dist_scale};
+                                              p.dist_scale, skip};
             march_loop(p.m, ry, smp, n_march, n_samp);
         } else {
             const float4* c4 = reinterpret_cast<const float4*>(p.cot + ray * kCotFloats);
@@ -343,6 +370,7 @@ __global__ void __launch_bounds__(128, NGPRT_BWD_MIN_BLOCKS) march_backward_kern
             BackwardSampler<L, AGG> smp{p.m.g, p.m.opts.attn_mode, p.m.opts.t_term, 1.0f, 0.0f, q2.y,
                                         {q0.x, q0.y, q0.z}, {q0.w, q1.x, q1.y, q1.z}, q1.w, q2.x, p.g_tables,
                                         p.g_coarse, slots, p.records, p.n_records, p.rec_capacity};
+            smp.skip = skip;
             march_loop(p.m, ry, smp, n_march, n_samp);
         }
     }

@@ -82,6 +82,7 @@ struct DistBwdSampler {
     float W_tot, S_tot, G_tot, scale;
     float* g_tables;
     float* g_coarse;
+    int skip;  // samples whose gradients are elsewhere already
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
         float f[8];
         sample_features<L, NGPRT_F32>(g, u, attn_mode, f, gates, blockDim.x);
@@ -96,7 +97,8 @@ struct DistBwdSampler {
         const float gw = 2.0f * (fmaf(m, W_lt, -S_lt) + (S_tot - S) - m * (W_tot - W)) + (2.0f / 3.0f) * w * delta;
         G = fmaf(w, gw, G);
         const float g_sigma = delta * (T_next * gw - (G_tot - G));
-        scatter_density<L>(g, u, attn_mode, scale * g_sigma * expf(fminf(f[0], 15.0f)), g_tables, g_coarse);
+        if (skip > 0) --skip;
+        else scatter_density<L>(g, u, attn_mode, scale * g_sigma * expf(fminf(f[0], 15.0f)), g_tables, g_coarse);
         T = T_next;
         return T < t_term;
     }
@@ -108,20 +110,50 @@ __global__ void __launch_bounds__(128) distortion_backward_kernel(const __grid_c
     int64_t ray;
     Ray ry;
     bool hit;
-    if (!ray_setup(p.m, ray, ry, hit)) return;
+    int skip = 0;
+    if (p.list) {
+        const int at = blockIdx.x * blockDim.x + threadIdx.x;
+        if (at >= *p.n_list) return;
+        ray = p.list[at].x;
+        skip = p.list[at].y;
+        hit = ray_setup_at(p.m, ray, ry);
+    } else if (!ray_setup(p.m, ray, ry, hit)) {
+        return;
+    }
     if (!hit) return;
     const float4 ds = reinterpret_cast<const float4*>(p.dist_state)[ray];
     DistBwdSampler<L> smp{p.m.g, p.m.opts.attn_mode, p.m.opts.t_term, gate_smem + threadIdx.x, 1.0f, 0.0f, 0.0f,
-                          0.0f, ds.y, ds.z, 2.0f * ds.x, p.scale, p.g_tables, p.g_coarse};
+                          0.0f, ds.y, ds.z, 2.0f * ds.x, p.scale, p.g_tables, p.g_coarse, skip};
     int n_march = 0, n_samp = 0;
     march_loop(p.m, ry, smp, n_march, n_samp);
 }
 
+// records: scratch of record_scratch_bytes (backward; p.m.plane is then set), or NULL.
 template <int L>
-void launch_dist(bool backward, const DistParams& p, dim3 grid, cudaStream_t st) {
+void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, cudaStream_t st) {
     const size_t shm = (size_t)2 * L * 128 * sizeof(float);
-    if (backward) distortion_backward_kernel<L><<<grid, 128, shm, st>>>(p);
-    else distortion_kernel<L, NGPRT_AGG_SEPARATE_V><<<grid, 128, shm, st>>>(p);
+    if (!backward) {
+        if (p.m.plane) distortion_plane_kernel<L><<<grid, 128, 0, st>>>(p);
+        else distortion_kernel<L, NGPRT_AGG_SEPARATE_V><<<grid, 128, shm, st>>>(p);
+        return;
+    }
+    if (!records) {
+        distortion_backward_kernel<L><<<grid, 128, shm, st>>>(p);
+        return;
+    }
+    RecParams r;
+    memset(&r, 0, sizeof r);
+    r.m = p.m;
+    r.dist_state = p.dist_state;
+    r.dist_scale = p.scale;
+    r.g_tables = p.g_tables;
+    r.g_coarse = p.g_coarse;
+    launch_records<L, true>(r, records, st, [&](const RecParams& q, unsigned blocks) {
+        DistParams rest = p;
+        rest.list = q.list;
+        rest.n_list = q.n_list;
+        distortion_backward_kernel<L><<<blocks, 128, shm, st>>>(rest);
+    });
 }
 
 }  // namespace
@@ -203,13 +235,23 @@ static int32_t run_distortion(bool backward, const ngprt_scene* scene, const ngp
         if (agg == NGPRT_AGG_MLP) launch_bwd_agg_mlp_wgrad(L, b, scene->agg_mlp, g_agg_mlp, st);
         return cuda_status(fn);
     }
+    void* records = nullptr;
+    if (workspace && plane_serves(scene)) {
+        const int64_t entries = ngprt_table_entries(scene);
+        const size_t plane = plane_layout(entries, backward ? 0 : n_rays).bytes;
+        const size_t rec = backward ? record_scratch_bytes(L, true, n_rays) : 0;
+        if (ws_bytes >= plane + rec && (!backward || rec)) {
+            density_scratch(p.m, entries, !backward, workspace, st);
+            if (backward) records = static_cast<char*>(workspace) + plane;
+        }
+    }
     switch (L) {
-        case 1: launch_dist<1>(backward, p, grid, st); break;
-        case 2: launch_dist<2>(backward, p, grid, st); break;
-        case 3: launch_dist<3>(backward, p, grid, st); break;
-        case 4: launch_dist<4>(backward, p, grid, st); break;
-        case 8: launch_dist<8>(backward, p, grid, st); break;
-        default: launch_dist<16>(backward, p, grid, st); break;
+        case 1: launch_dist<1>(backward, p, grid, records, st); break;
+        case 2: launch_dist<2>(backward, p, grid, records, st); break;
+        case 3: launch_dist<3>(backward, p, grid, records, st); break;
+        case 4: launch_dist<4>(backward, p, grid, records, st); break;
+        case 8: launch_dist<8>(backward, p, grid, records, st); break;
+        default: launch_dist<16>(backward, p, grid, records, st); break;
     }
     return cuda_status(fn);
 }
@@ -222,8 +264,18 @@ extern "C" int32_t ngprt_distortion_loss(const ngprt_scene* scene, const ngprt_o
                                          int32_t n_cams, const int32_t* pixel_ids, const float* rays_o,
                                          const float* rays_d, int64_t n_rays, const ngprt_render_opts* opts,
                                          float scale, float* dist_state, float* loss, void* stream) {
+    return ngprt_distortion_loss_ws(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n_rays, opts, scale, dist_state,
+                                    loss, nullptr, 0, stream);
+}
+
+extern "C" int32_t ngprt_distortion_loss_ws(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
+                                            int32_t n_cams, const int32_t* pixel_ids, const float* rays_o,
+                                            const float* rays_d, int64_t n_rays, const ngprt_render_opts* opts,
+                                            float scale, float* dist_state, float* loss, void* workspace,
+                                            size_t ws_bytes, void* stream) {
     return run_distortion(false, scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n_rays, opts, dist_state, scale,
-                          loss, nullptr, nullptr, nullptr, nullptr, nullptr, 0, stream, "ngprt_distortion_loss");
+                          loss, nullptr, nullptr, nullptr, nullptr, workspace, ws_bytes, stream,
+                          "ngprt_distortion_loss");
 }
 
 extern "C" size_t ngprt_distortion_backward_workspace_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
@@ -231,6 +283,14 @@ extern "C" size_t ngprt_distortion_backward_workspace_bytes(const ngprt_scene* s
     if (!scene || n_rays < 0 || scene->aggregation != NGPRT_AGG_MLP) return 0;
     const int64_t ms = opts && opts->max_samples > 0 ? opts->max_samples : 0;
     return 256 + (size_t)n_rays * (size_t)ms * (size_t)(kNFeat * (scene->L + 1)) * sizeof(float);
+}
+
+extern "C" size_t ngprt_distortion_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
+                                                          int64_t n_rays) {
+    const size_t b = ngprt_distortion_backward_workspace_bytes(scene, opts, n_rays);
+    if (n_rays < 0 || !plane_serves(scene)) return b;
+    const size_t rec = record_scratch_bytes(scene->L, true, n_rays);
+    return rec ? plane_layout(ngprt_table_entries(scene), 0).bytes + rec : b;
 }
 
 extern "C" int32_t ngprt_distortion_backward(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,

@@ -2,7 +2,7 @@
 // on the aggregation form: distortion.cu builds Eq. 8, distortion_agg.cu the other
 // forms of Table 3 (whose reverse pass is the reverse march in distortion mode).
 #pragma once
-#include "backward_march.cuh"
+#include "records.cuh"
 
 namespace ngprt {
 
@@ -13,11 +13,13 @@ struct DistParams {
     float* loss;
     float* g_tables;
     float* g_coarse;
+    const int2* list;        // backward: only these rays, from these samples on (NULL: all)
+    const int32_t* n_list;
 };
 
-template <int L, int AGG>
+template <class Weights>
 struct DistSampler {
-    ForwardSampler<L, NGPRT_F32, AGG> fw;
+    Weights fw;
     float W, S, Lp, Ls;
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
         const bool stop = fw.sample(u, t, delta);
@@ -31,18 +33,15 @@ struct DistSampler {
     }
 };
 
-template <int L, int AGG>
-__global__ void __launch_bounds__(128) distortion_kernel(const __grid_constant__ DistParams p) {
-    extern __shared__ float gate_smem[];
+template <class Weights>
+__device__ __forceinline__ void distortion_ray(const DistParams& p, const Weights& weights) {
     int64_t ray = 0;
     Ray ry;
     bool hit = false;
     const bool has_ray = ray_setup(p.m, ray, ry, hit);
     float Ld = 0.0f;
     if (has_ray) {
-        DistSampler<L, AGG> smp{ForwardSampler<L, NGPRT_F32, AGG>(p.m.g, p.m.opts.attn_mode, p.m.opts.t_term,
-                                                                  gate_smem + threadIdx.x),
-                                0.0f, 0.0f, 0.0f, 0.0f};
+        DistSampler<Weights> smp{weights, 0.0f, 0.0f, 0.0f, 0.0f};
         int n_march = 0, n_samp = 0;
         if (hit) march_loop(p.m, ry, smp, n_march, n_samp);
         Ld = smp.Lp + smp.Ls;
@@ -55,6 +54,19 @@ __global__ void __launch_bounds__(128) distortion_kernel(const __grid_constant__
         for (int k = 16; k > 0; k >>= 1) v += __shfl_xor_sync(0xffffffffu, v, k);
         if ((threadIdx.x & 31) == 0 && v != 0.0f) atomicAdd(p.loss, p.scale * v);
     }
+}
+
+template <int L, int AGG>
+__global__ void __launch_bounds__(128) distortion_kernel(const __grid_constant__ DistParams p) {
+    extern __shared__ float gate_smem[];
+    distortion_ray(p, ForwardSampler<L, NGPRT_F32, AGG>(p.m.g, p.m.opts.attn_mode, p.m.opts.t_term,
+                                                        gate_smem + threadIdx.x));
+}
+
+// The same from the density channel alone (p.m.plane).
+template <int L>
+__global__ void __launch_bounds__(128, kWeightMinBlocks) distortion_plane_kernel(const __grid_constant__ DistParams p) {
+    distortion_ray(p, WeightSampler<L>(p.m.g, p.m.plane, p.m.opts.attn_mode, p.m.opts.t_term));
 }
 
 // The forms of Table 3 other than Eq. 8 (distortion_agg.cu): L = 2, 4, 16.

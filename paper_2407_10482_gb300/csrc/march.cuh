@@ -48,6 +48,8 @@ struct MarchParams {
     int32_t* stats;
     const float* fb_a_hat;  // fallback pass: predicted opacity per ray (NULL otherwise)
     float fb_thr;           // re-march a ray when a_hat - A(interval) > fb_thr
+    const int32_t* perm;    // order in which a ray list is taken (NULL: as given)
+    const float* plane;     // the tables' density channel (sample_density), or NULL
     // camera tiles handed out at run time (zeroed before the launch), or NULL: each
     // warp takes the tile of its own index
     unsigned long long* tile_counter;
@@ -76,6 +78,7 @@ __device__ __forceinline__ bool thread_ray(const MarchParams& p, int64_t& ray, f
     }
     ray = tile_of_warp >= 0 ? tile_of_warp * 32 + lane : (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (ray >= p.n_rays) return false;
+    if (p.perm) ray = p.perm[ray];
     if (p.mode == 1) {
         int64_t id = p.pixel_ids[ray];
         if (id < 0) id = 0;
@@ -248,7 +251,9 @@ __device__ __forceinline__ void level_gates(const Grid& g, uint32_t cb, uint32_t
 // colour channels of f^l times gq (the ray's colour cotangents) in the slots
 // gates[(2L + 2l) * stride] and gates[(2L + 2l + 1) * stride]; the MLP form leaves
 // f^l in the slots [8l, 8l + 8) and its 64 hidden pre-activations in [8L, 8L + 64).
-template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V, bool kKeep = false>
+// With kRec (the reverse pass's records, Eq. 8), gates is the record's level fields and
+// every level leaves omega^l, beta^l, sigma^l and q^l in its four.
+template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V, bool kKeep = false, bool kRec = false>
 __device__ __forceinline__ void sample_features(const Grid& g, const float u[3], int attn_mode, float f[8],
                                                 float* gates, int stride, const float* gq = nullptr) {
     constexpr int NC = coarse_channels(L, AGG);
@@ -419,6 +424,17 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
                 for (int ch = 0; ch < 4; ++ch) fl[ch] = ffma2(cw2, make_float2(e[c][2 * ch], e[c][2 * ch + 1]), fl[ch]);
             }
         }
+        static_assert(!kRec || kFly, "records take the gates level by level");
+        [[maybe_unused]] float q_l = 0.0f;
+        if constexpr (kRec) {
+            q_l = fl[0].y * gq[0];
+            q_l = fmaf(fl[1].x, gq[1], q_l);
+            q_l = fmaf(fl[1].y, gq[2], q_l);
+            q_l = fmaf(fl[2].x, gq[3], q_l);
+            q_l = fmaf(fl[2].y, gq[4], q_l);
+            q_l = fmaf(fl[3].x, gq[5], q_l);
+            q_l = fmaf(fl[3].y, gq[6], q_l);
+        }
         if constexpr (kKeep && AGG == NGPRT_AGG_MLP) {
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
@@ -467,6 +483,12 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
                 om = gates[(2 * l) * stride];
                 be = gates[(2 * l + 1) * stride];
             }
+            if constexpr (kRec) {
+                gates[(4 * l) * stride] = om;
+                gates[(4 * l + 1) * stride] = be;
+                gates[(4 * l + 2) * stride] = fl[0].x;
+                gates[(4 * l + 3) * stride] = q_l;
+            }
 #pragma unroll
             for (int ch = 0; ch < 4; ++ch) {
                 const float2 r = ffma2(make_float2(ch == 0 ? om : be, be), fl[ch], make_float2(f[2 * ch], f[2 * ch + 1]));
@@ -506,6 +528,81 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
             f[k] += o;
         }
     }
+}
+
+// ------------------------------------------------------------- the density path alone
+//
+// The passes that need nothing but the samples' weights (the distortion regulariser, the
+// visibility marks, the density occupancy) read one of an FP32 entry's eight channels.  A
+// 4-byte load of it moves the entry's whole 32-byte sector from L2 all the same, and at
+// about 180 G sectors a second that is what bounds them (reading 4 bytes in place of 32
+// from the tables themselves gained nothing: hd, 4 views of 960 x 540, 12.7 ms either
+// way).  So the density channel is copied to a plane of its own first (hd: 25 MB, which
+// L2 holds, against 191 MB, which it does not; 35 us): eight neighbouring rows
+// share a sector, the two x corners of a cell mostly do.
+
+// f[0] of sample_features for FP32 Eq. 8 scenes, bit for bit: the same products and sums
+// in the same order.  plane: the tables' channel 0, one float per row.  With kRec each
+// level leaves omega^l and sigma^l in rec[(2l) * 32] and rec[(2l + 1) * 32].
+template <int L, bool kRec = false>
+__device__ __forceinline__ float sample_density(const Grid& g, const float* __restrict__ plane, const float u[3],
+                                                int attn_mode, float* rec = nullptr) {
+    constexpr int NC = coarse_channels(L, NGPRT_AGG_SEPARATE_V);
+    int b[3];
+    float w[3];
+#pragma unroll
+    for (int a = 0; a < 3; ++a) grid_cell(u[a], g.R_C, b[a], w[a]);
+    uint32_t cb, sy, sz;
+    coarse_base(g, b, cb, sy, sz);
+    float ccw[8];
+    const float* row[8];
+    float f0 = 0.0f;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const uint32_t v = cb + (uint32_t)(c & 1) + sy * (uint32_t)((c >> 1) & 1) + sz * (uint32_t)((c >> 2) & 1);
+        row[c] = static_cast<const float*>(g.coarse) + (size_t)v * NC;
+        ccw[c] = corner_w(w, c);
+        f0 = fmaf(ccw[c], __ldg(row[c]), f0);
+    }
+    auto level = [&](const int l, auto kind) {
+        constexpr int kKind = decltype(kind)::value;
+        int bl[3];
+        float wl[3];
+#pragma unroll
+        for (int a = 0; a < 3; ++a) grid_cell(u[a], g.N[l], bl[a], wl[a]);
+        const float* tl = plane + g.level_off[l];
+        float q[8];
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+            q[c] = __ldg(tl + level_index_k<kKind>(g, l, (uint32_t)(bl[0] + (c & 1)), (uint32_t)(bl[1] + ((c >> 1) & 1)),
+                                                   (uint32_t)(bl[2] + ((c >> 2) & 1))));
+        float om = 1.0f;
+        if (attn_mode != 1) {
+            float lg = 0.0f;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) lg = fmaf(ccw[c], __ldg(row[c] + kNFeat + 2 * l), lg);
+            om = gate_sigmoid(lg);
+        }
+        float sg = 0.0f;
+#pragma unroll
+        for (int c = 0; c < 8; ++c) sg = fmaf(corner_w(wl, c), q[c], sg);
+        if constexpr (kRec) {
+            rec[(2 * l) * 32] = om;
+            rec[(2 * l + 1) * 32] = sg;
+        }
+        f0 = fmaf(om, sg, f0);
+    };
+    if (g.n_dense >= 0) {
+        const int nd = min(g.n_dense, L);
+#pragma unroll 1
+        for (int l = 0; l < nd; ++l) level(l, std::integral_constant<int, 1>{});
+#pragma unroll 1
+        for (int l = nd; l < L; ++l) level(l, std::integral_constant<int, 2>{});
+    } else {
+#pragma unroll 1
+        for (int l = 0; l < L; ++l) level(l, std::integral_constant<int, 0>{});
+    }
+    return f0;
 }
 
 // Shared-memory floats per thread that sample_features parks its gates in (forward
@@ -780,6 +877,30 @@ struct ForwardSampler {
         float f[8];
         sample_features<L, DT, AGG>(g, u, attn_mode, f, gates, blockDim.x);
         return composite(f, t, delta);
+    }
+};
+
+// Blocks per SM of the marches on sample_density (hd, visibility of 4 views of 960 x 540
+// with the rest of the pipeline: 7.85 ms at 7, 8.03 at 6, 8.53 at 5, 8.33 at 9).
+constexpr int kWeightMinBlocks = 7;
+
+// The forward's weights without its features: w and T of every sample exactly as
+// ForwardSampler composites them.
+template <int L>
+struct WeightSampler {
+    const Grid& g;
+    const float* plane;
+    int attn_mode;
+    float t_term;
+    float T = 1.0f, w_last = 0.0f;
+    __device__ __forceinline__ WeightSampler(const Grid& g_, const float* plane_, int mode, float term)
+        : g(g_), plane(plane_), attn_mode(mode), t_term(term) {}
+    __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
+        const float sigma = expf(sample_density<L>(g, plane, u, attn_mode));
+        const float trans = expf(-sigma * delta);
+        w_last = T * (1.0f - trans);
+        T *= trans;
+        return T < t_term;
     }
 };
 

@@ -3,6 +3,7 @@
 // voxels of samples whose weight passes a threshold), and box dilation.  The
 // pyramid and the distance grid G of the result then come from ngprt_build_occ_dist.
 #include "occupancy.cuh"
+#include "records.cuh"
 
 namespace ngprt {
 
@@ -37,8 +38,19 @@ static bool pow2_in(int32_t R) { return R >= 2 && R <= 1024 && (R & (R - 1)) == 
 
 using namespace ngprt;
 
+extern "C" size_t ngprt_density_scratch_bytes(const ngprt_scene* scene, int64_t n_rays) {
+    if (n_rays < 0 || !plane_serves(scene)) return 0;
+    return plane_layout(ngprt_table_entries(scene), n_rays).bytes;
+}
+
 extern "C" int32_t ngprt_occupancy_from_density(const ngprt_scene* scene, const ngprt_render_opts* opts, int32_t R,
                                                 float sigma_thr, uint8_t* occ_out, float* sigma_out, void* stream) {
+    return ngprt_occupancy_from_density_ws(scene, opts, R, sigma_thr, occ_out, sigma_out, nullptr, 0, stream);
+}
+
+extern "C" int32_t ngprt_occupancy_from_density_ws(const ngprt_scene* scene, const ngprt_render_opts* opts, int32_t R,
+                                                   float sigma_thr, uint8_t* occ_out, float* sigma_out, void* workspace,
+                                                   size_t ws_bytes, void* stream) {
     const char* fn = "ngprt_occupancy_from_density";
     DensityOccParams p;
     memset(&p, 0, sizeof p);
@@ -59,6 +71,14 @@ extern "C" int32_t ngprt_occupancy_from_density(const ngprt_scene* scene, const 
         launch_density_agg(scene->L, scene->aggregation, scene->table_dtype, p, st);
         return cuda_status(fn);
     }
+    const bool built = scene->L <= 4 || scene->L == 8 || scene->L == 16;
+    if (built && workspace && plane_serves(scene) && ws_bytes >= ngprt_density_scratch_bytes(scene, 0)) {
+        MarchParams m;
+        memset(&m, 0, sizeof m);
+        m.g = p.g;
+        density_scratch(m, ngprt_table_entries(scene), false, workspace, st);
+        p.plane = m.plane;
+    }
     switch (scene->L) {
         case 1: launch_density<1, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, st); break;
         case 2: launch_density<2, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, st); break;
@@ -76,6 +96,15 @@ extern "C" int32_t ngprt_occupancy_visibility(const ngprt_scene* scene, const ng
                                               const float* rays_o, const float* rays_d, int64_t n_rays,
                                               const ngprt_render_opts* opts, float w_thr, int32_t R, uint8_t* vis,
                                               void* stream) {
+    return ngprt_occupancy_visibility_ws(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n_rays, opts, w_thr, R,
+                                         vis, nullptr, 0, stream);
+}
+
+extern "C" int32_t ngprt_occupancy_visibility_ws(const ngprt_scene* scene, const ngprt_occ* occ,
+                                                 const ngprt_camera* cams, int32_t n_cams, const int32_t* pixel_ids,
+                                                 const float* rays_o, const float* rays_d, int64_t n_rays,
+                                                 const ngprt_render_opts* opts, float w_thr, int32_t R, uint8_t* vis,
+                                                 void* workspace, size_t ws_bytes, void* stream) {
     const char* fn = "ngprt_occupancy_visibility";
     MarchParams p;
     memset(&p, 0, sizeof p);
@@ -97,6 +126,9 @@ extern "C" int32_t ngprt_occupancy_visibility(const ngprt_scene* scene, const ng
         launch_visibility_agg(scene->L, scene->aggregation, scene->table_dtype, p, grid, w_thr, R, vis, st);
         return cuda_status(fn);
     }
+    const bool built = scene->L <= 4 || scene->L == 8 || scene->L == 16;
+    if (built && workspace && plane_serves(scene) && ws_bytes >= ngprt_density_scratch_bytes(scene, n_rays))
+        density_scratch(p, ngprt_table_entries(scene), true, workspace, st);
     switch (scene->L) {
         case 1: launch_visibility<1, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, grid, w_thr, R, vis, st); break;
         case 2: launch_visibility<2, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, grid, w_thr, R, vis, st); break;

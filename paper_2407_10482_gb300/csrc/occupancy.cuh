@@ -14,10 +14,12 @@ struct DensityOccParams {
     float sigma_thr;
     uint8_t* occ;
     float* sigma;
+    const float* plane;  // the tables' density channel, or NULL
 };
 
-// One voxel per thread: sigma = exp(sigma_raw) at the voxel centre (Eq. 6-8).
-template <int L, int DT, int AGG>
+// One voxel per thread: sigma = exp(sigma_raw) at the voxel centre (Eq. 6-8); kPlane: on
+// the density channel alone.
+template <int L, int DT, int AGG, bool kPlane = false>
 __global__ void __launch_bounds__(128) density_occ_kernel(const __grid_constant__ DensityOccParams p) {
     extern __shared__ float gate_smem[];
     const int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -28,7 +30,8 @@ __global__ void __launch_bounds__(128) density_occ_kernel(const __grid_constant_
     const float u[3] = {fmul(fadd((float)i, 0.5f), inv), fmul(fadd((float)j, 0.5f), inv),
                         fmul(fadd((float)k, 0.5f), inv)};
     float f[8];
-    sample_features<L, DT, AGG>(p.g, u, p.attn_mode, f, gate_smem + threadIdx.x, blockDim.x);
+    if constexpr (kPlane) f[0] = sample_density<L>(p.g, p.plane, u, p.attn_mode);
+    else sample_features<L, DT, AGG>(p.g, u, p.attn_mode, f, gate_smem + threadIdx.x, blockDim.x);
     const float sg = expf(f[0]);
     p.occ[v] = sg > p.sigma_thr ? 1 : 0;
     if (p.sigma) p.sigma[v] = sg;
@@ -36,9 +39,9 @@ __global__ void __launch_bounds__(128) density_occ_kernel(const __grid_constant_
 
 // Composites like the forward render and marks the voxel (R^3 grid) of every sample
 // whose weight exceeds w_thr.  All writers store 1, so concurrent marks agree.
-template <int L, int DT, int AGG>
+template <class Weights>
 struct VisibilitySampler {
-    ForwardSampler<L, DT, AGG> fw;
+    Weights fw;
     float w_thr;
     int32_t R;
     uint8_t* vis;
@@ -61,8 +64,22 @@ __global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
     bool hit;
     extern __shared__ float gate_smem[];
     if (!ray_setup(p, ray, ry, hit)) return;
-    VisibilitySampler<L, DT, AGG> smp{
+    VisibilitySampler<ForwardSampler<L, DT, AGG>> smp{
         ForwardSampler<L, DT, AGG>(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x), w_thr, R, vis};
+    int n_march = 0, n_samp = 0;
+    if (hit) march_loop(p, ry, smp, n_march, n_samp);
+}
+
+// The same marks from the density channel alone (p.plane).
+template <int L>
+__global__ void __launch_bounds__(128, kWeightMinBlocks)
+    visibility_plane_kernel(const __grid_constant__ MarchParams p, float w_thr, int32_t R, uint8_t* vis) {
+    int64_t ray;
+    Ray ry;
+    bool hit;
+    if (!ray_setup(p, ray, ry, hit)) return;
+    VisibilitySampler<WeightSampler<L>> smp{WeightSampler<L>(p.g, p.plane, p.opts.attn_mode, p.opts.t_term), w_thr, R,
+                                            vis};
     int n_march = 0, n_samp = 0;
     if (hit) march_loop(p, ry, smp, n_march, n_samp);
 }
@@ -71,6 +88,12 @@ template <int L, int AGG>
 void launch_density(int dt, const DensityOccParams& p, cudaStream_t st) {
     const int64_t n = (int64_t)p.R * p.R * p.R;
     const unsigned blocks = (unsigned)((n + 127) / 128);
+    if constexpr (AGG == NGPRT_AGG_SEPARATE_V) {
+        if (p.plane) {
+            density_occ_kernel<L, NGPRT_F32, AGG, true><<<blocks, 128, 0, st>>>(p);
+            return;
+        }
+    }
     const size_t shm = (size_t)2 * L * 128 * sizeof(float);
     if (dt == NGPRT_F32) density_occ_kernel<L, NGPRT_F32, AGG><<<blocks, 128, shm, st>>>(p);
     else if (dt == NGPRT_F16) density_occ_kernel<L, NGPRT_F16, AGG><<<blocks, 128, shm, st>>>(p);
@@ -80,6 +103,12 @@ void launch_density(int dt, const DensityOccParams& p, cudaStream_t st) {
 template <int L, int AGG>
 void launch_visibility(int dt, const MarchParams& p, dim3 grid, float w_thr, int32_t R, uint8_t* vis,
                        cudaStream_t st) {
+    if constexpr (AGG == NGPRT_AGG_SEPARATE_V) {
+        if (p.plane) {
+            visibility_plane_kernel<L><<<grid, 128, 0, st>>>(p, w_thr, R, vis);
+            return;
+        }
+    }
     const size_t shm = (size_t)2 * L * 128 * sizeof(float);
     if (dt == NGPRT_F32) visibility_kernel<L, NGPRT_F32, AGG><<<grid, 128, shm, st>>>(p, w_thr, R, vis);
     else if (dt == NGPRT_F16) visibility_kernel<L, NGPRT_F16, AGG><<<grid, 128, shm, st>>>(p, w_thr, R, vis);

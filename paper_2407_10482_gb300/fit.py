@@ -95,9 +95,10 @@ def tile_order(pixel_ids: torch.Tensor, W: int, H: int, tile: int = 32):
     """(perm, inv): the permutation that groups a minibatch's pixel ids by view and
     tile x tile image tile (row-major inside a tile), and its inverse.  The render
     runs fastest on rays in this order (neighbouring lanes sample neighbouring
-    points); the reverse pass runs fastest in the drawn random order (neighbouring
-    lanes then rarely add gradients to the same entries), so the state moves back
-    through inv between the two."""
+    points); the reverse pass takes large batches of camera pixels in such an order by
+    itself, whatever order it is given, and small ones run fastest in the drawn order
+    (neighbouring lanes then rarely add gradients to the same entries), so the state
+    moves back through inv between the two."""
     p = pixel_ids.long()
     v, rem = p // (W * H), p % (W * H)
     row, col = rem // W, rem % W

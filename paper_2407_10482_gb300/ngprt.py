@@ -70,9 +70,16 @@ _SIGS = {
     "ngprt_occupancy_from_density": (C.c_int32, [_P, _P, C.c_int32, C.c_float, _P, _P, _P]),
     "ngprt_occupancy_visibility": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, C.c_float,
                                                C.c_int32, _P, _P]),
+    "ngprt_density_scratch_bytes": (C.c_size_t, [_P, C.c_int64]),
+    "ngprt_occupancy_from_density_ws": (C.c_int32, [_P, _P, C.c_int32, C.c_float, _P, _P, _P, C.c_size_t, _P]),
+    "ngprt_occupancy_visibility_ws": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, C.c_float,
+                                                  C.c_int32, _P, _P, C.c_size_t, _P]),
     "ngprt_huber_loss": (C.c_int32, [_P, _P, C.c_int64, C.c_float, C.c_float, _P, _P, _P]),
     "ngprt_distortion_loss": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, C.c_float, _P, _P,
                                           _P]),
+    "ngprt_distortion_loss_ws": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, C.c_float, _P, _P, _P,
+                                             C.c_size_t, _P]),
+    "ngprt_distortion_backward_scratch_bytes": (C.c_size_t, [_P, _P, C.c_int64]),
     "ngprt_distortion_backward": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, _P, C.c_float,
                                               _P, _P, _P, _P, _P, C.c_size_t, _P]),
     "ngprt_distortion_backward_workspace_bytes": (C.c_size_t, [_P, _P, C.c_int64]),
@@ -89,6 +96,7 @@ _SIGS = {
                                  _P, C.c_size_t, _P]),
     "ngprt_render_backward": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, _P, _P, _P, _P,
                                           _P, _P, _P, _P, _P, _P, C.c_size_t, _P]),
+    "ngprt_render_backward_scratch_bytes": (C.c_size_t, [_P, _P, C.c_int64]),
     "ngprt_render_backward_workspace_bytes": (C.c_size_t, [_P, _P, C.c_int64]),
     "ngprt_grid_indices": (C.c_int32, [_P, _P, C.c_int64, _P, _P]),
     "ngprt_shade": (C.c_int32, [_P, _P, C.c_int64, _P, _P, _P, _P, _P]),
@@ -157,6 +165,22 @@ def _stream(stream=None) -> int | None:
     return stream.cuda_stream
 
 
+def _scratch(nbytes: int, like: torch.Tensor, stream=None):
+    """Scratch of a call that also runs without any: a block of torch's caching allocator
+    on the call's stream, or None (nothing to gain, no memory left, a capture running)."""
+    if not nbytes:
+        return None
+    if stream is not None:
+        with torch.cuda.stream(stream):
+            return _scratch(nbytes, like)
+    if torch.cuda.is_current_stream_capturing():
+        return None
+    try:
+        return torch.empty(nbytes, dtype=torch.uint8, device=like.device)
+    except torch.OutOfMemoryError:
+        return None
+
+
 def _check(fn: str, rc: int) -> None:
     if rc != OK:
         raise NgprtError(fn, rc, lib().ngprt_last_error().decode())
@@ -188,15 +212,18 @@ def ngprt_coarse_channels(L: int, aggregation: int) -> int:
 
 
 def ngprt_occupancy_from_density(scene, opts, R, sigma_thr, occ_out, sigma_out=None, stream=None) -> None:
-    _check("ngprt_occupancy_from_density", lib().ngprt_occupancy_from_density(
-        C.byref(scene), C.byref(opts), R, sigma_thr, _ptr(occ_out), _ptr(sigma_out), _stream(stream)))
+    ws = _scratch(ngprt_density_scratch_bytes(scene, 0), occ_out, stream)
+    _check("ngprt_occupancy_from_density", lib().ngprt_occupancy_from_density_ws(
+        C.byref(scene), C.byref(opts), R, sigma_thr, _ptr(occ_out), _ptr(sigma_out), _ptr(ws),
+        ws.numel() if ws is not None else 0, _stream(stream)))
 
 
 def ngprt_occupancy_visibility(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n_rays, opts, w_thr, R, vis,
                                stream=None) -> None:
-    _check("ngprt_occupancy_visibility", lib().ngprt_occupancy_visibility(
+    ws = _scratch(ngprt_density_scratch_bytes(scene, n_rays), vis, stream)
+    _check("ngprt_occupancy_visibility", lib().ngprt_occupancy_visibility_ws(
         C.byref(scene), C.byref(occ), cams, n_cams, _ptr(pixel_ids), _ptr(rays_o), _ptr(rays_d), n_rays,
-        C.byref(opts), w_thr, R, _ptr(vis), _stream(stream)))
+        C.byref(opts), w_thr, R, _ptr(vis), _ptr(ws), ws.numel() if ws is not None else 0, _stream(stream)))
 
 
 def ngprt_huber_loss(rgb, target, n, delta, scale, loss=None, d_rgb=None, stream=None) -> None:
@@ -206,14 +233,18 @@ def ngprt_huber_loss(rgb, target, n, delta, scale, loss=None, d_rgb=None, stream
 
 def ngprt_distortion_loss(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n_rays, opts, scale, dist_state,
                           loss=None, stream=None) -> None:
-    _check("ngprt_distortion_loss", lib().ngprt_distortion_loss(
+    ws = _scratch(ngprt_density_scratch_bytes(scene, n_rays), dist_state, stream)
+    _check("ngprt_distortion_loss", lib().ngprt_distortion_loss_ws(
         C.byref(scene), C.byref(occ), cams, n_cams, _ptr(pixel_ids), _ptr(rays_o), _ptr(rays_d), n_rays,
-        C.byref(opts), scale, _ptr(dist_state), _ptr(loss), _stream(stream)))
+        C.byref(opts), scale, _ptr(dist_state), _ptr(loss), _ptr(ws), ws.numel() if ws is not None else 0,
+        _stream(stream)))
 
 
 def ngprt_distortion_backward(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n_rays, opts, dist_state, scale,
                               g_tables, g_coarse, stream=None, g_attn_inv=None, g_agg_mlp=None,
                               workspace=None) -> None:
+    if workspace is None and not ngprt_distortion_backward_workspace_bytes(scene, opts, n_rays):
+        workspace = _scratch(ngprt_distortion_backward_scratch_bytes(scene, opts, n_rays), g_tables, stream)
     ws_bytes = workspace.numel() * workspace.element_size() if workspace is not None else 0
     _check("ngprt_distortion_backward", lib().ngprt_distortion_backward(
         C.byref(scene), C.byref(occ), cams, n_cams, _ptr(pixel_ids), _ptr(rays_o), _ptr(rays_d), n_rays,
@@ -223,6 +254,14 @@ def ngprt_distortion_backward(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_
 
 def ngprt_distortion_backward_workspace_bytes(scene, opts, n_rays) -> int:
     return int(lib().ngprt_distortion_backward_workspace_bytes(C.byref(scene), C.byref(opts), n_rays))
+
+
+def ngprt_distortion_backward_scratch_bytes(scene, opts, n_rays) -> int:
+    return int(lib().ngprt_distortion_backward_scratch_bytes(C.byref(scene), C.byref(opts), n_rays))
+
+
+def ngprt_density_scratch_bytes(scene, n_rays) -> int:
+    return int(lib().ngprt_density_scratch_bytes(C.byref(scene), n_rays))
 
 
 def ngprt_mean_samples(ray_stats, n_rays, out, stream=None) -> None:
@@ -294,6 +333,10 @@ def ngprt_render_backward(scene, occ, cams, n_cams, pixel_ids, rays_o, rays_d, n
 
 def ngprt_render_backward_workspace_bytes(scene, opts, n_rays) -> int:
     return int(lib().ngprt_render_backward_workspace_bytes(C.byref(scene), C.byref(opts), n_rays))
+
+
+def ngprt_render_backward_scratch_bytes(scene, opts, n_rays) -> int:
+    return int(lib().ngprt_render_backward_scratch_bytes(C.byref(scene), C.byref(opts), n_rays))
 
 
 def coarse_blocks_per_axis(R_C: int) -> int:
@@ -568,8 +611,12 @@ def _renderer_backward(self, opts, state, d_rgb, d_depth, d_opacity, g_tables, g
         cam_arr, n_cams = None, 0
         n = rays_o.shape[0]
     ro = render_opts(opts)
-    need = ngprt_render_backward_workspace_bytes(self.scene.struct, ro, n)
-    if self._bws is None or self._bws.numel() < need:
+    best = ngprt_render_backward_scratch_bytes(self.scene.struct, ro, n)
+    if self._bws is None or self._bws.numel() < best:
+        self._bws = None  # given back before a larger one is asked for
+        self._bws = _scratch(best, self.scene.tables)
+    if self._bws is None:
+        need = ngprt_render_backward_workspace_bytes(self.scene.struct, ro, n)
         self._bws = torch.empty(need, dtype=torch.uint8, device=self.device)
     ngprt_render_backward(self.scene.struct, self.occ.struct, cam_arr, n_cams, pixel_ids, rays_o, rays_d, n,
                           ro, state, d_rgb, d_depth, d_opacity, g_tables, g_coarse, g_mlp, self._bws,
