@@ -319,6 +319,25 @@ static __global__ void plane_kernel(const float* __restrict__ tables, int64_t n,
     }
 }
 
+// Atomic, as every addition to the gradients: another stream may add to them too.
+static __global__ void add_plane_kernel(const float* __restrict__ plane, int64_t n, float* __restrict__ g_tables) {
+    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= n) return;
+    const float v = __ldg(plane + i);
+    if (v != 0.0f) atomicAdd(g_tables + 8 * i, v);
+}
+
+float* gradient_plane(int64_t entries, void* scratch, cudaStream_t st) {
+    char* base = reinterpret_cast<char*>(((uintptr_t)scratch + 255) & ~(uintptr_t)255);
+    float* plane = reinterpret_cast<float*>(base + plane_layout(entries, 0, true).grad);
+    cudaMemsetAsync(plane, 0, (size_t)entries * sizeof(float), st);
+    return plane;
+}
+
+void add_gradient_plane(const float* plane, int64_t entries, float* g_tables, cudaStream_t st) {
+    add_plane_kernel<<<(unsigned)((entries + 255) / 256), 256, 0, st>>>(plane, entries, g_tables);
+}
+
 void density_scratch(MarchParams& p, int64_t entries, bool order, void* scratch, cudaStream_t st) {
     const PlaneLayout a = plane_layout(entries, order ? p.n_rays : 0);
     char* base = reinterpret_cast<char*>(((uintptr_t)scratch + 255) & ~(uintptr_t)255);
@@ -326,7 +345,10 @@ void density_scratch(MarchParams& p, int64_t entries, bool order, void* scratch,
     plane_kernel<<<(unsigned)((entries + 1023) / 1024), 256, 0, st>>>(static_cast<const float*>(p.g.tables), entries, plane);
     p.plane = plane;
     p.perm = nullptr;
-    if (order && p.n_rays >= kRecordMinRays && p.n_rays <= 0x7FFFFFFF)
+    if (!order) return;
+    p.tile_counter = reinterpret_cast<unsigned long long*>(base + a.counter);
+    cudaMemsetAsync(p.tile_counter, 0, sizeof(unsigned long long), st);
+    if (p.n_rays >= kRecordMinRays && p.n_rays <= 0x7FFFFFFF)
         p.perm = bin_rays(p, reinterpret_cast<uint32_t*>(base + a.bins), reinterpret_cast<int32_t*>(base + a.perm), st);
 }
 

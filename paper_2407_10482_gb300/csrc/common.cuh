@@ -76,6 +76,7 @@ __device__ __forceinline__ float fadd(float a, float b) { return __fadd_rn(a, b)
 __device__ __forceinline__ float fsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ float fmul(float a, float b) { return __fmul_rn(a, b); }
 __device__ __forceinline__ float fdiv(float a, float b) { return __fdiv_rn(a, b); }
+__device__ __forceinline__ float frcp(float a) { return __frcp_rn(a); }  // fdiv(1, a), cheaper
 __device__ __forceinline__ float fsqrt(float a) { return __fsqrt_rn(a); }
 
 // ------------------------------------------------ double-float (hi + lo) values
@@ -215,9 +216,10 @@ __device__ __forceinline__ bool ray_interval(int bounded, const float o[3], cons
 
 // World position x = o + t d at the double-float parameter t (products by
 // two-product, one final rounding of the correction), its radius r, the
-// contracted point y (mip-NeRF 360 when unbounded) and the unit-cube coordinate u.
+// contracted point y (mip-NeRF 360 when unbounded) and the unit-cube coordinate u;
+// beyond the unit ball ir = 1 / r and k = (2 - 1/r) / r (else 0 and 1).
 __device__ __forceinline__ void march_point(int bounded, const Ray& ry, df t, float x[3], float y[3], float u[3],
-                                            float& r) {
+                                            float& r, float& ir, float& k) {
 #pragma unroll
     for (int a = 0; a < 3; ++a) {
         const df q = df_prod(t.hi, ry.dh[a]);
@@ -226,9 +228,11 @@ __device__ __forceinline__ void march_point(int bounded, const Ray& ry, df t, fl
         x[a] = fadd(s.hi, corr);
     }
     r = fsqrt(dot3(x, x));
+    ir = 0.0f;
+    k = 1.0f;
     if (!bounded && r > 1.0f) {
-        const float ir = fdiv(1.0f, r);
-        const float k = fmul(fsub(2.0f, ir), ir);  // (2 - 1/r) / r
+        ir = frcp(r);
+        k = fmul(fsub(2.0f, ir), ir);
 #pragma unroll
         for (int a = 0; a < 3; ++a) y[a] = fmul(x[a], k);
     } else {

@@ -128,13 +128,19 @@ __global__ void __launch_bounds__(128) distortion_backward_kernel(const __grid_c
     march_loop(p.m, ry, smp, n_march, n_samp);
 }
 
-// records: scratch of record_scratch_bytes (backward; p.m.plane is then set), or NULL.
+// records: scratch of record_scratch_bytes (backward; p.m.plane and g_plane are then
+// set), or NULL.
 template <int L>
-void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, cudaStream_t st) {
+void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, float* g_plane, cudaStream_t st) {
     const size_t shm = (size_t)2 * L * 128 * sizeof(float);
     if (!backward) {
-        if (p.m.plane) distortion_plane_kernel<L><<<grid, 128, 0, st>>>(p);
-        else distortion_kernel<L, NGPRT_AGG_SEPARATE_V><<<grid, 128, shm, st>>>(p);
+        if (p.m.plane) {
+            static int cache[16] = {0};
+            const unsigned most = resident_grid(distortion_plane_kernel<L>, cache);
+            distortion_plane_kernel<L><<<grid.x < most ? grid.x : most, 128, 0, st>>>(p);
+            return;
+        }
+        distortion_kernel<L, NGPRT_AGG_SEPARATE_V><<<grid, 128, shm, st>>>(p);
         return;
     }
     if (!records) {
@@ -148,6 +154,7 @@ void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, c
     r.dist_scale = p.scale;
     r.g_tables = p.g_tables;
     r.g_coarse = p.g_coarse;
+    r.g_plane = g_plane;
     launch_records<L, true>(r, records, st, [&](const RecParams& q, unsigned blocks) {
         DistParams rest = p;
         rest.list = q.list;
@@ -236,23 +243,28 @@ static int32_t run_distortion(bool backward, const ngprt_scene* scene, const ngp
         return cuda_status(fn);
     }
     void* records = nullptr;
+    float* g_plane = nullptr;
     if (workspace && plane_serves(scene)) {
         const int64_t entries = ngprt_table_entries(scene);
-        const size_t plane = plane_layout(entries, backward ? 0 : n_rays).bytes;
+        const size_t plane = plane_layout(entries, backward ? 0 : n_rays, backward).bytes;
         const size_t rec = backward ? record_scratch_bytes(L, true, n_rays) : 0;
         if (ws_bytes >= plane + rec && (!backward || rec)) {
             density_scratch(p.m, entries, !backward, workspace, st);
-            if (backward) records = static_cast<char*>(workspace) + plane;
+            if (backward) {
+                records = static_cast<char*>(workspace) + plane;
+                g_plane = gradient_plane(entries, workspace, st);
+            }
         }
     }
     switch (L) {
-        case 1: launch_dist<1>(backward, p, grid, records, st); break;
-        case 2: launch_dist<2>(backward, p, grid, records, st); break;
-        case 3: launch_dist<3>(backward, p, grid, records, st); break;
-        case 4: launch_dist<4>(backward, p, grid, records, st); break;
-        case 8: launch_dist<8>(backward, p, grid, records, st); break;
-        default: launch_dist<16>(backward, p, grid, records, st); break;
+        case 1: launch_dist<1>(backward, p, grid, records, g_plane, st); break;
+        case 2: launch_dist<2>(backward, p, grid, records, g_plane, st); break;
+        case 3: launch_dist<3>(backward, p, grid, records, g_plane, st); break;
+        case 4: launch_dist<4>(backward, p, grid, records, g_plane, st); break;
+        case 8: launch_dist<8>(backward, p, grid, records, g_plane, st); break;
+        default: launch_dist<16>(backward, p, grid, records, g_plane, st); break;
     }
+    if (g_plane) add_gradient_plane(g_plane, ngprt_table_entries(scene), g_tables, st);
     return cuda_status(fn);
 }
 
@@ -290,7 +302,7 @@ extern "C" size_t ngprt_distortion_backward_scratch_bytes(const ngprt_scene* sce
     const size_t b = ngprt_distortion_backward_workspace_bytes(scene, opts, n_rays);
     if (n_rays < 0 || !plane_serves(scene)) return b;
     const size_t rec = record_scratch_bytes(scene->L, true, n_rays);
-    return rec ? plane_layout(ngprt_table_entries(scene), 0).bytes + rec : b;
+    return rec ? plane_layout(ngprt_table_entries(scene), 0, true).bytes + rec : b;
 }
 
 extern "C" int32_t ngprt_distortion_backward(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,

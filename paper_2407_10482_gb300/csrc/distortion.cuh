@@ -34,11 +34,11 @@ struct DistSampler {
 };
 
 template <class Weights>
-__device__ __forceinline__ void distortion_ray(const DistParams& p, const Weights& weights) {
+__device__ __forceinline__ void distortion_ray(const DistParams& p, const Weights& weights, int64_t tile = -1) {
     int64_t ray = 0;
     Ray ry;
     bool hit = false;
-    const bool has_ray = ray_setup(p.m, ray, ry, hit);
+    const bool has_ray = ray_setup(p.m, ray, ry, hit, tile);
     float Ld = 0.0f;
     if (has_ray) {
         DistSampler<Weights> smp{weights, 0.0f, 0.0f, 0.0f, 0.0f};
@@ -63,10 +63,13 @@ __global__ void __launch_bounds__(128) distortion_kernel(const __grid_constant__
                                                         gate_smem + threadIdx.x));
 }
 
-// The same from the density channel alone (p.m.plane).
+// The same from the density channel alone (p.m.plane), tiles handed out at run time.
 template <int L>
 __global__ void __launch_bounds__(128, kWeightMinBlocks) distortion_plane_kernel(const __grid_constant__ DistParams p) {
-    distortion_ray(p, WeightSampler<L>(p.m.g, p.m.plane, p.m.opts.attn_mode, p.m.opts.t_term));
+    for (int64_t tile; (tile = next_tile(p.m)) >= 0;) {
+        distortion_ray(p, WeightSampler<L>(p.m.g, p.m.plane, p.m.opts.attn_mode, p.m.opts.t_term), tile);
+        __syncwarp();
+    }
 }
 
 // The forms of Table 3 other than Eq. 8 (distortion_agg.cu): L = 2, 4, 16.

@@ -651,11 +651,10 @@ __device__ __forceinline__ MarchState march_state(const Ray& ry) {
     return st;
 }
 
-// Image speed J(x) d of the contraction along the ray (r = |x| > 1):
+// Image speed J(x) d of the contraction along the ray (r = |x| > 1, ir = 1 / r):
 // J d = k d + m x with k = (2 - 1/r)/r and m = (x.d) 2 (1 - r) / r^4.
-__device__ __forceinline__ void contracted_dir(const float x[3], const float d[3], float r, float v[3]) {
-    const float ir = fdiv(1.0f, r);
-    const float kk = fmul(fsub(2.0f, ir), ir);
+__device__ __forceinline__ void contracted_dir(const float x[3], const float d[3], float r, float ir, float kk,
+                                               float v[3]) {
     const float px = dot3(x, d);
     const float ir2 = fmul(ir, ir);
     const float m = fmul(fmul(px, fmul(2.0f, fsub(1.0f, r))), fmul(ir2, ir2));
@@ -667,23 +666,22 @@ __device__ __forceinline__ void contracted_dir(const float x[3], const float d[3
 // past the exit face of its voxel.
 constexpr float kEmptyGuard = 0.02f;
 
-// s_O (Sec. 3.3): the step that leaves empty voxel ev of resolution Rk.  The image
+// s_O (Sec. 3.3): the step that leaves empty voxel ev of side vk (2B / R_k; g: the guard in
+// the same units; ir, kk: march_point's).  The image
 // of the ray is aimed at the plane kEmptyGuard finest voxels (side 2B / R_O) beyond
 // the voxel's exit face: along the image's local direction v = J(x) d first, which
 // picks the exit axis; beyond the unit ball the image curves, and one Newton step on
 // that axis, from the image's position and direction at the first estimate (the
 // correction clamped to half of it), corrects the length.
 __device__ __forceinline__ float empty_step(int bounded, const float x[3], const float y[3], const float d[3],
-                                            float r, const int ev[3], int Rk, int R_O) {
+                                            float r, float ir, float kk, const int ev[3], float vk, float g) {
     const float B = bounded ? 1.0f : 2.0f;
     const bool curved = !bounded && r > 1.0f;
     float v[3];
-    if (curved) contracted_dir(x, d, r, v);
+    if (curved) contracted_dir(x, d, r, ir, kk, v);
     else {
         v[0] = d[0]; v[1] = d[1]; v[2] = d[2];
     }
-    const float vk = fdiv(2.0f * B, (float)Rk);
-    const float g = fmul(kEmptyGuard, fdiv(2.0f * B, (float)R_O));
     // the exit axis's values are carried by selection (no array indexed at run time)
     float s0 = INFINITY, target = 0.0f, v_ax = 0.0f, d_ax = 0.0f, x_ax = 0.0f;
 #pragma unroll
@@ -713,12 +711,12 @@ __device__ __forceinline__ float empty_step(int bounded, const float x[3], const
     const float r1 = fsqrt(dot3(x1, x1));
     float y1, v1;
     if (r1 > 1.0f) {
-        const float ir = fdiv(1.0f, r1);
-        const float kk = fmul(fsub(2.0f, ir), ir);
-        const float ir2 = fmul(ir, ir);
+        const float ir1 = frcp(r1);
+        const float kk1 = fmul(fsub(2.0f, ir1), ir1);
+        const float ir2 = fmul(ir1, ir1);
         const float m = fmul(fmul(dot3(x1, d), fmul(2.0f, fsub(1.0f, r1))), fmul(ir2, ir2));
-        y1 = fmul(x1_ax, kk);
-        v1 = fadd(fmul(kk, d_ax), fmul(m, x1_ax));
+        y1 = fmul(x1_ax, kk1);
+        v1 = fadd(fmul(kk1, d_ax), fmul(m, x1_ax));
     } else {
         y1 = x1_ax;
         v1 = d_ax;
@@ -742,11 +740,14 @@ __device__ __forceinline__ bool march_advance(const MarchParams& p, const Ray& r
     const int R_O = p.occ.R_O;
     const int R_G = p.occ.R_G;
     const float vG = fdiv(2.0f * B, (float)R_G);
+    // side of a finest voxel, a power of two: a level's is its exact multiple
+    const float v0 = fdiv(2.0f * B, (float)R_O);
+    const float guard = fmul(kEmptyGuard, v0);
     const bool snap = op.lattice_snap && bounded;
     while (df_lt(st.t, st.t_out) && st.n_march < op.max_march && st.n_samp < op.max_samples) {
         ++st.n_march;
-        float x[3], y[3], r;
-        march_point(bounded, ry, st.t, x, y, u, r);
+        float x[3], y[3], r, ir, kc;
+        march_point(bounded, ry, st.t, x, y, u, r, ir, kc);
         int empty_level = -1, ev[3] = {0, 0, 0};
         // the finest level's voxel, once: R_O is a power of two, so u R_k = u R_O / 2^k
         // exactly and a coarser level's voxel is the finest one's shifted right by k
@@ -767,7 +768,7 @@ __device__ __forceinline__ bool march_advance(const MarchParams& p, const Ray& r
             delta = fminf(dt, fadd(fsub(st.t_out.hi, st.t.hi), fsub(st.t_out.lo, st.t.lo)));
             return true;
         }
-        const float s_O = empty_step(bounded, x, y, ry.dh, r, ev, R_O >> empty_level, R_O);
+        const float s_O = empty_step(bounded, x, y, ry.dh, r, ir, kc, ev, fmul(v0, (float)(1 << empty_level)), guard);
         float step = s_O;
         if (op.use_dist && p.occ.dist && empty_level > p.occ.g_shift) {
             const int gs = p.occ.g_shift;
@@ -826,6 +827,16 @@ __device__ __forceinline__ void march_loop(const MarchParams& p, const Ray& ry, 
     march_loop_from(p, ry, st, smp);
     n_march = st.n_march;
     n_samp = st.n_samp;
+}
+
+// The next tile (camera tile or run of 32 rays) of a warp that takes them from
+// p.tile_counter until none are left; -1 when there is none.
+__device__ __forceinline__ int64_t next_tile(const MarchParams& p) {
+    const int64_t tiles = p.mode == 0 ? (int64_t)p.tiles_per_view * p.n_cams : (p.n_rays + 31) / 32;
+    unsigned long long t = 0;
+    if ((threadIdx.x & 31) == 0) t = atomicAdd(p.tile_counter, 1ull);
+    t = __shfl_sync(0xffffffffu, t, 0);
+    return t < (unsigned long long)tiles ? (int64_t)t : -1;
 }
 
 // Forward sampler: features (Eq. 6-8), alpha compositing (Eq. 2, Eq. 5).
@@ -980,14 +991,8 @@ __global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
         one_ray(-1);
         return;
     }
-    const int64_t tiles = p.mode == 0 ? (int64_t)p.tiles_per_view * p.n_cams : (p.n_rays + 31) / 32;
-    const int lane = threadIdx.x & 31;
-    for (;;) {
-        unsigned long long t = 0;
-        if (lane == 0) t = atomicAdd(p.tile_counter, 1ull);
-        t = __shfl_sync(0xffffffffu, t, 0);
-        if (t >= (unsigned long long)tiles) break;
-        one_ray((int64_t)t);
+    for (int64_t tile; (tile = next_tile(p)) >= 0;) {
+        one_ray(tile);
         __syncwarp();
     }
 }
@@ -1077,6 +1082,16 @@ int resident_blocks(Kernel k, size_t shm) {
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per, k, 128, shm);
     return (sms > 0 ? sms : 1) * (per > 0 ? per : 1);
+}
+
+// The same without shared memory, found once per device (cache: 16 zeros at first).
+template <class Kernel>
+unsigned resident_grid(Kernel k, int* cache) {
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev < 0 || dev >= 16) dev = 0;
+    if (!cache[dev]) cache[dev] = resident_blocks(k, 0);
+    return (unsigned)cache[dev];
 }
 
 template <int L, int DT, int AGG>

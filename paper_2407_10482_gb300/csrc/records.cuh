@@ -22,17 +22,20 @@
 // step of the warp is one slot of a chunk of kSlots steps x 32 lanes, taken from a
 // counter when the previous chunk is full.  Record fields are lane-contiguous:
 //     u (3), gs, w, then omega, beta, sigma^l, q^l per level   (kDist: u, gs, omega, sigma^l)
-// Kernel 2 (scatter_kernel): one warp per (job, chunk), a job being a level, the coarse
-// feature channels or a group of coarse logits; job-major, so that one level's gradient
-// rows (16.7 MB for a hashed hd level) stay in L2 while all chunks add to them.
+// Kernel 2 (scatter_levels_kernel, scatter_logits_kernel): one warp per (job, chunk), a
+// job being a level, the coarse feature channels or a group of coarse logits; job-major,
+// so that one level's gradient rows (16.7 MB for a hashed hd level) stay in L2 while all
+// chunks add to them.
 // Rays whose records find no chunk left go to a list (with their first unrecorded
 // sample) that the one-kernel form finishes.
 //
-// hd scene, 2^18 camera pixels of 8 views: march 3.4 ms (4 blocks per SM; 3.8 at 5, where
-// it spills) + scatter 4.8 ms in place of 21.0 ms in one kernel.  The scatter was 7.0 ms
-// with 8 steps a chunk and each lane adding its rows by itself, 6.4 with 16 steps; pairing
-// the lanes gave the rest.  The march is bound by the same 180 G sectors a second that its
-// gathers take from L2.  The regulariser at the same rays: 1.9 + 3.6 ms in place of 29.3.
+// hd scene, 2^18 camera pixels of 8 views: march 3.3 ms (4 blocks per SM; 3.8 at 5, where
+// it spills) + scatter 4.4 ms in place of 21.0 ms in one kernel.  The scatter was 7.0 ms
+// with 8 steps a chunk and each lane adding its rows by itself, 6.4 with 16 steps, 4.8 with
+// the lanes in pairs; levels and logits in kernels of their own, each with the blocks its
+// registers allow, gave the rest.  The march is bound by the same 180 G sectors a second
+// that its gathers take from L2.  The regulariser at the same rays: 1.9 + 2.8 ms in place
+// of 29.3 (3.6 for the scatter before it had a gradient plane).
 #pragma once
 #include <string.h>
 
@@ -62,6 +65,7 @@ struct RecParams {
     float dist_scale;
     float* g_tables;
     float* g_coarse;
+    float* g_plane;           // distortion: the density channel's gradient, one float per row
     float* rec;               // [max_chunks][kSlots][fields][32]
     int32_t* chunk_ray;       // [max_chunks][32] ray of each lane
     int32_t* chunk_n;         // [max_chunks][32] records of each lane
@@ -138,8 +142,8 @@ __global__ void __launch_bounds__(128, kDist ? 6 : 4) record_kernel(const __grid
                 r[64] = u[2];
                 float f[8];
                 if constexpr (kDist) f[0] = sample_density<L, true>(p.m.g, p.m.plane, u, p.m.opts.attn_mode, r + 4 * 32);
-                else sample_features<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V, false, true>(p.m.g, u, p.m.opts.attn_mode, f,
-                                                                                      r + 5 * 32, 32, gq);
+                else sample_features<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V, false, true>(
+                    p.m.g, u, p.m.opts.attn_mode, f, r + 5 * 32, 32, gq);
                 const float t = df_float(st.t);
                 const float sigma = expf(f[0]);
                 const float trans = expf(-sigma * delta);
@@ -189,23 +193,43 @@ __device__ __forceinline__ void add_row(float* p, const float* v) {
     }
 }
 
-// Levels per logit group of the coarse grid: 8 channels' sums at 8 corners.
-template <bool kDist>
-constexpr int logit_levels() {
-    return kDist ? 8 : 4;
+// Adds the halves of 8-float rows with the two lanes of a pair side by side: a row is one
+// sector, and the pair adds the two halves of one lane's row in the same instruction, then
+// of the other's, so that L2 gets one request per row and not one per half.  row: this
+// lane's (kNoRow: none); mine, theirs: the half (even lanes the first, odd lanes the
+// second) of this lane's row and of its neighbour's.
+constexpr uint32_t kNoRow = 0xFFFFFFFFu;
+template <int kAlign>
+__device__ __forceinline__ void add_pair(float* grid, uint32_t row, size_t row_floats, const float* mine,
+                                         const float* theirs) {
+    const bool odd = threadIdx.x & 1;
+    const uint32_t other = __shfl_xor_sync(0xffffffffu, row, 1);
+    float* half = grid + (odd ? 4 : 0);
+    const uint32_t r1 = odd ? other : row, r2 = odd ? row : other;
+    if (r1 != kNoRow) add_row<4, kAlign>(half + r1 * row_floats, odd ? theirs : mine);
+    if (r2 != kNoRow) add_row<4, kAlign>(half + r2 * row_floats, odd ? mine : theirs);
 }
 
+__device__ __forceinline__ uint32_t vertex_row(const int b[3], int c, uint32_t N) {
+    return (uint32_t)(b[0] + (c & 1)) + N * ((uint32_t)(b[1] + ((c >> 1) & 1)) + N * (uint32_t)(b[2] + ((c >> 2) & 1)));
+}
+
+// Scatter of the levels and of the coarse feature channels (job L: omega = beta = 1).  One
+// warp per (job, chunk), a lane per ray.  The next record is loaded while the present one
+// is added; 6 blocks per SM (2^18 pixels of the hd scene, forward and reverse pass: 12.62 ms
+// against 12.66 at 7, 12.87 at 8 and 14.5 at 10, where it spills).
+// kDist adds to a plane of the density gradient (hd: 25 MB, all of it in L2): the rows of
+// two x neighbours are one 8-byte reduction there where they are an aligned pair (every
+// hashed cell with an even x, and every other dense one).
 template <int L, bool kDist>
-__global__ void __launch_bounds__(128, 4) scatter_kernel(const __grid_constant__ RecParams p) {
+__global__ void __launch_bounds__(128, kDist ? 8 : 6) scatter_levels_kernel(const __grid_constant__ RecParams p) {
     constexpr int F = record_floats<L, kDist>();
     constexpr int NC = kNFeat + 2 * L;
-    constexpr int kGroup = logit_levels<kDist>();
-    constexpr int kLf = kDist ? 4 : 5;  // first level field
+    constexpr int kLf = kDist ? 4 : 5, kPer = kDist ? 2 : 4;  // first level field, fields a level
     const Grid& g = p.m.g;
     const int lane = threadIdx.x & 31;
     const uint32_t n_chunks = min(*p.n_chunks, p.max_chunks);
-    const int jobs = L + 1 + (p.m.opts.attn_mode == 1 ? 0 : (L + kGroup - 1) / kGroup);
-    const uint64_t items = (uint64_t)jobs * n_chunks;
+    const uint64_t items = (uint64_t)(L + 1) * n_chunks;
     const uint64_t n_warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
     for (uint64_t it = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += n_warps) {
         const int job = (int)(it / n_chunks);
@@ -213,148 +237,201 @@ __global__ void __launch_bounds__(128, 4) scatter_kernel(const __grid_constant__
         const int n = p.chunk_n[(size_t)chunk * 32 + lane];
         const int n_max = __reduce_max_sync(0xffffffffu, n);
         const float* rec = p.rec + (size_t)chunk * (kSlots * F * 32) + lane;
-        int pb[3] = {-1, -1, -1};
-        if (job <= L) {
-            // a level, or the coarse feature channels (job L: omega = beta = 1)
-            const bool coarse = job == L;
-            const int N = coarse ? g.R_C : g.N[job];
-            float* const grid = coarse ? p.g_coarse : p.g_tables + (size_t)g.level_off[job] * 8;
-            // cotangents of the row half that this lane adds (even lanes channels 0-3,
-            // odd lanes 4-7): of its own ray and of its neighbour's
-            float own[4] = {0.0f, 0.0f, 0.0f, 0.0f}, nbr[4] = {0.0f, 0.0f, 0.0f, 0.0f};
-            if constexpr (!kDist) {
-                const float* c = p.cot + (int64_t)p.chunk_ray[(size_t)chunk * 32 + lane] * kCotFloats;
-                const float* cn = p.cot + (int64_t)p.chunk_ray[(size_t)chunk * 32 + (lane ^ 1)] * kCotFloats;
+        const bool coarse = job == L;
+        const int N = coarse ? g.R_C : g.N[job];
+        float* const grid = coarse ? p.g_coarse : kDist ? p.g_plane : p.g_tables + (size_t)g.level_off[job] * 8;
+        // cotangents of the row half that this lane adds (even lanes channels 0-3, odd
+        // lanes 4-7): of its own ray and of its neighbour's
+        float own[4] = {0.0f, 0.0f, 0.0f, 0.0f}, nbr[4] = {0.0f, 0.0f, 0.0f, 0.0f};
+        if constexpr (!kDist) {
+            const float* c = p.cot + (int64_t)p.chunk_ray[(size_t)chunk * 32 + lane] * kCotFloats;
+            const float* cn = p.cot + (int64_t)p.chunk_ray[(size_t)chunk * 32 + (lane ^ 1)] * kCotFloats;
 #pragma unroll
-                for (int k = 0; k < 4; ++k) {
-                    // floats 0-6 of the record are the cotangents of channels 1-7
-                    if (lane & 1) {
-                        own[k] = c[3 + k];
-                        nbr[k] = cn[3 + k];
-                    } else if (k > 0) {
-                        own[k] = c[k - 1];
-                        nbr[k] = cn[k - 1];
-                    }
+            for (int k = 0; k < 4; ++k) {
+                // floats 0-6 of the record are the cotangents of channels 1-7
+                if (lane & 1) {
+                    own[k] = c[3 + k];
+                    nbr[k] = cn[3 + k];
+                } else if (k > 0) {
+                    own[k] = c[k - 1];
+                    nbr[k] = cn[k - 1];
                 }
             }
-            float sa[8], sb[8];
+        }
+        float sa[8], sb[8];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) sa[c] = sb[c] = 0.0f;
-            // Adds the sums of the lanes with `go` to their 8 rows.  A row of 8 floats is
-            // one sector: the two lanes of a pair add the halves of one lane's row in the
-            // same instruction, then of the other's, so that L2 gets one request per row
-            // and not one per half.
-            auto flush = [&](bool go) {
-                if (!__any_sync(0xffffffffu, go)) return;
+        for (int c = 0; c < 8; ++c) sa[c] = sb[c] = 0.0f;
+        int pb[3] = {-1, -1, -1};
+        // adds the sums of the lanes with `go` to their 8 rows
+        auto flush = [&](bool go) {
+            if (!__any_sync(0xffffffffu, go)) return;
+            auto row_of = [&](int c) {
+                return coarse ? vertex_row(pb, c, (uint32_t)N)
+                              : level_index(g, job, (uint32_t)(pb[0] + (c & 1)), (uint32_t)(pb[1] + ((c >> 1) & 1)),
+                                            (uint32_t)(pb[2] + ((c >> 2) & 1)));
+            };
+            if constexpr (kDist) {
+                if (!go) return;
+#pragma unroll
+                for (int c = 0; c < 8; c += 2) {
+                    if (coarse) {
+                        atomicAdd(grid + (size_t)row_of(c) * NC, sa[c]);
+                        atomicAdd(grid + (size_t)row_of(c + 1) * NC, sa[c + 1]);
+                        continue;
+                    }
+                    const uint32_t r0 = g.level_off[job] + row_of(c), r1 = g.level_off[job] + row_of(c + 1);
+                    if ((r0 ^ r1) == 1u) {
+                        const bool swap = r0 & 1u;
+                        atomicAdd(reinterpret_cast<float2*>(grid + (r0 & ~1u)),
+                                  make_float2(swap ? sa[c + 1] : sa[c], swap ? sa[c] : sa[c + 1]));
+                    } else {
+                        atomicAdd(grid + r0, sa[c]);
+                        atomicAdd(grid + r1, sa[c + 1]);
+                    }
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) sa[c] = 0.0f;
+            } else {
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const uint32_t x = (uint32_t)(pb[0] + (c & 1)), y = (uint32_t)(pb[1] + ((c >> 1) & 1)),
-                                   z = (uint32_t)(pb[2] + ((c >> 2) & 1));
-                    const uint32_t row = coarse ? x + (uint32_t)N * (y + (uint32_t)N * z) : level_index(g, job, x, y, z);
-                    if constexpr (kDist) {
-                        if (go) atomicAdd(grid + (size_t)row * (coarse ? NC : 8), sa[c]);
-                    } else {
-                        const uint32_t mine = go ? row : 0xFFFFFFFFu;
-                        const uint32_t theirs = __shfl_xor_sync(0xffffffffu, mine, 1);
-                        const float an = __shfl_xor_sync(0xffffffffu, sa[c], 1), bn = __shfl_xor_sync(0xffffffffu, sb[c], 1);
-                        const bool odd = lane & 1;
-                        const float v[4] = {odd ? sb[c] * own[0] : sa[c], sb[c] * own[1], sb[c] * own[2], sb[c] * own[3]};
-                        const float vn[4] = {odd ? bn * nbr[0] : an, bn * nbr[1], bn * nbr[2], bn * nbr[3]};
-                        const uint32_t r1 = odd ? theirs : mine, r2 = odd ? mine : theirs;
-                        const int half = odd ? 4 : 0;
-                        auto add = [&](uint32_t r, const float* h) {
-                            if (r == 0xFFFFFFFFu) return;
-                            if (coarse) add_row<4, NC>(grid + (size_t)r * NC + half, h);
-                            else add_row<4, 8>(grid + (size_t)r * 8 + half, h);
-                        };
-                        add(r1, odd ? vn : v);
-                        add(r2, odd ? v : vn);
-                    }
+                    const uint32_t row = go ? row_of(c) : kNoRow;
+                    const float an = __shfl_xor_sync(0xffffffffu, sa[c], 1), bn = __shfl_xor_sync(0xffffffffu, sb[c], 1);
+                    const bool odd = lane & 1;
+                    const float v[4] = {odd ? sb[c] * own[0] : sa[c], sb[c] * own[1], sb[c] * own[2], sb[c] * own[3]};
+                    const float vn[4] = {odd ? bn * nbr[0] : an, bn * nbr[1], bn * nbr[2], bn * nbr[3]};
+                    if (coarse) add_pair<NC>(grid, row, NC, v, vn);
+                    else add_pair<8>(grid, row, 8, v, vn);
                     if (go) sa[c] = sb[c] = 0.0f;
                 }
-            };
-#pragma unroll 1
-            for (int k = 0; k < n_max; ++k) {
-                const bool on = k < n;
-                int b[3] = {pb[0], pb[1], pb[2]};
-                float w[3], a = 0.0f, bw = 0.0f;
-                if (on) {
-                    const float* r = rec + k * (F * 32);
-                    const float u[3] = {r[0], r[32], r[64]};
-                    a = r[96];
-                    if constexpr (!kDist) bw = r[128];
-                    if (!coarse) {
-                        a *= r[(kLf + (kDist ? 2 : 4) * job) * 32];
-                        if constexpr (!kDist) bw *= r[(kLf + 4 * job + 1) * 32];
-                    }
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) grid_cell(u[d], N, b[d], w[d]);
-                }
-                const bool moved = b[0] != pb[0] || b[1] != pb[1] || b[2] != pb[2];
-                flush(moved && k > 0);
-                if (on) {
-                    pb[0] = b[0]; pb[1] = b[1]; pb[2] = b[2];
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const float cw = corner_w(w, c);
-                        sa[c] = fmaf(cw, a, sa[c]);
-                        if constexpr (!kDist) sb[c] = fmaf(cw, bw, sb[c]);
-                    }
-                }
             }
-            flush(n > 0);
-        } else {
-            // the logits of levels l0 .. l0 + kGroup - 1 at the coarse vertices
-            if (n == 0) continue;
-            const int l0 = (job - L - 1) * kGroup;
-            constexpr int NV = 8;
-            const int mode = p.m.opts.attn_mode;
-            const int R = g.R_C;
-            float s[8][NV];
+        };
+        // u, gs and w times the level's omega and beta of record k
+        float u[3] = {0.0f, 0.0f, 0.0f}, x[4] = {0.0f, 0.0f, 1.0f, 1.0f};
+        auto load = [&](int k) {
+            if (k >= n) return;
+            const float* r = rec + k * (F * 32);
+            u[0] = r[0];
+            u[1] = r[32];
+            u[2] = r[64];
+            x[0] = r[96];
+            if constexpr (!kDist) x[1] = r[128];
+            if (!coarse) {
+                x[2] = r[(kLf + kPer * job) * 32];
+                if constexpr (!kDist) x[3] = r[(kLf + kPer * job + 1) * 32];
+            }
+        };
+        load(0);
+#pragma unroll 1
+        for (int k = 0; k < n_max; ++k) {
+            const bool on = k < n;
+            int b[3];
+            float w[3];
 #pragma unroll
-            for (int c = 0; c < 8; ++c)
-#pragma unroll
-                for (int v = 0; v < NV; ++v) s[c][v] = 0.0f;
-            auto flush = [&]() {
+            for (int d = 0; d < 3; ++d) grid_cell(u[d], N, b[d], w[d]);
+            const float a = x[0] * x[2], bw = x[1] * x[3];
+            load(k + 1);
+            const bool moved = on && (b[0] != pb[0] || b[1] != pb[1] || b[2] != pb[2]);
+            flush(moved && k > 0);
+            if (on) {
+                pb[0] = b[0]; pb[1] = b[1]; pb[2] = b[2];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
-                    const uint32_t x = (uint32_t)(pb[0] + (c & 1)), y = (uint32_t)(pb[1] + ((c >> 1) & 1)),
-                                   z = (uint32_t)(pb[2] + ((c >> 2) & 1));
-                    float* gp = p.g_coarse + (size_t)(x + (uint32_t)R * (y + (uint32_t)R * z)) * NC + kNFeat + 2 * l0;
-                    if constexpr (kDist && L % 8 == 0) {
-                        // the omega logits are every other channel: a zero added to the
-                        // beta logit between two of them costs less than a second request
+                    const float cw = corner_w(w, c);
+                    sa[c] = fmaf(cw, a, sa[c]);
+                    if constexpr (!kDist) sb[c] = fmaf(cw, bw, sb[c]);
+                }
+            }
+        }
+        flush(n > 0);
+    }
+}
+
+// Scatter of the coarse logits, kGroup levels at a time: 8 channels' sums at 8 corners.
+template <int L, bool kDist>
+__global__ void __launch_bounds__(128, 4) scatter_logits_kernel(const __grid_constant__ RecParams p) {
+    constexpr int F = record_floats<L, kDist>();
+    constexpr int NC = kNFeat + 2 * L;
+    constexpr int kGroup = kDist ? 8 : 4;
+    constexpr int kLf = kDist ? 4 : 5, kPer = kDist ? 2 : 4;
+    constexpr int NV = 8;
+    const Grid& g = p.m.g;
+    const int lane = threadIdx.x & 31, mode = p.m.opts.attn_mode, R = g.R_C;
+    const uint32_t n_chunks = min(*p.n_chunks, p.max_chunks);
+    const uint64_t items = (uint64_t)((L + kGroup - 1) / kGroup) * n_chunks;
+    const uint64_t n_warps = (uint64_t)gridDim.x * (blockDim.x >> 5);
+    for (uint64_t it = ((uint64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5; it < items; it += n_warps) {
+        const int l0 = (int)(it / n_chunks) * kGroup;
+        const uint32_t chunk = (uint32_t)(it % n_chunks);
+        const int n = p.chunk_n[(size_t)chunk * 32 + lane];
+        const int n_max = __reduce_max_sync(0xffffffffu, n);
+        const float* rec = p.rec + (size_t)chunk * (kSlots * F * 32) + lane;
+        float* const grid = p.g_coarse + kNFeat + 2 * l0;
+        float s[8][NV];
 #pragma unroll
-                        for (int v = 0; v < NV; v += 2) atomic_add4(gp + 2 * v, s[c][v], 0.0f, s[c][v + 1], 0.0f);
-                    } else if constexpr (kDist) {
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+            for (int v = 0; v < NV; ++v) s[c][v] = 0.0f;
+        int pb[3] = {-1, -1, -1};
+        auto flush = [&](bool go) {
+            if (!__any_sync(0xffffffffu, go)) return;
+            const bool odd = lane & 1;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) {
+                const uint32_t row = go ? vertex_row(pb, c, (uint32_t)R) : kNoRow;
+                if constexpr (!kDist && L % 4 == 0) {
+                    float mine[4], theirs[4];
+#pragma unroll
+                    for (int v = 0; v < 4; ++v) {
+                        mine[v] = odd ? s[c][4 + v] : s[c][v];
+                        theirs[v] = __shfl_xor_sync(0xffffffffu, odd ? s[c][v] : s[c][4 + v], 1);
+                    }
+                    add_pair<NC>(grid, row, NC, mine, theirs);
+                } else if constexpr (kDist && L % 8 == 0) {
+                    // the omega logits are every other channel; a zero added to the beta
+                    // logit between two of them costs less than a second request
+#pragma unroll
+                    for (int h = 0; h < 2; ++h) {
+                        const float* q = s[c] + 4 * h;
+                        const float mine[4] = {odd ? q[2] : q[0], 0.0f, odd ? q[3] : q[1], 0.0f};
+                        const float theirs[4] = {__shfl_xor_sync(0xffffffffu, odd ? q[0] : q[2], 1), 0.0f,
+                                                 __shfl_xor_sync(0xffffffffu, odd ? q[1] : q[3], 1), 0.0f};
+                        add_pair<NC>(grid + 8 * h, row, NC, mine, theirs);
+                    }
+                } else if (go) {
+                    float* gp = grid + (size_t)row * NC;
+                    if constexpr (kDist) {
 #pragma unroll
                         for (int v = 0; v < NV; ++v)
                             if (v < L && l0 + v < L) atomicAdd(gp + 2 * v, s[c][v]);
-                    } else if constexpr (L % kGroup == 0) {
-                        add_row<NV, NC>(gp, s[c]);
                     } else {
 #pragma unroll
                         for (int v = 0; v < NV; v += 2)
                             if (v / 2 < L && l0 + v / 2 < L)
                                 atomicAdd(reinterpret_cast<float2*>(gp + v), make_float2(s[c][v], s[c][v + 1]));
                     }
+                }
+                if (go) {
 #pragma unroll
                     for (int v = 0; v < NV; ++v) s[c][v] = 0.0f;
                 }
-            };
+            }
+        };
 #pragma unroll 1
-            for (int k = 0; k < n; ++k) {
+        for (int k = 0; k < n_max; ++k) {
+            const bool on = k < n;
+            int b[3] = {pb[0], pb[1], pb[2]};
+            float w[3] = {0.0f, 0.0f, 0.0f}, val[NV];
+#pragma unroll
+            for (int v = 0; v < NV; ++v) val[v] = 0.0f;
+            if (on) {
                 const float* r = rec + k * (F * 32);
                 const float u[3] = {r[0], r[32], r[64]};
                 const float gs = r[96];
                 const float w_ = kDist ? 0.0f : r[128];
-                float val[NV];
-#pragma unroll
-                for (int v = 0; v < NV; ++v) val[v] = 0.0f;
 #pragma unroll
                 for (int j = 0; j < kGroup; ++j) {
                     if (j >= L || l0 + j >= L) continue;
-                    const float* q = r + (kLf + (kDist ? 2 : 4) * (l0 + j)) * 32;
+                    const float* q = r + (kLf + kPer * (l0 + j)) * 32;
                     if constexpr (kDist) {
                         const float om = q[0], sh = q[32];
                         val[j] = gs * sh * om * (1.0f - om);
@@ -368,14 +445,13 @@ __global__ void __launch_bounds__(128, 4) scatter_kernel(const __grid_constant__
                         }
                     }
                 }
-                int b[3];
-                float w[3];
 #pragma unroll
                 for (int d = 0; d < 3; ++d) grid_cell(u[d], R, b[d], w[d]);
-                if (b[0] != pb[0] || b[1] != pb[1] || b[2] != pb[2]) {
-                    if (k > 0) flush();
-                    pb[0] = b[0]; pb[1] = b[1]; pb[2] = b[2];
-                }
+            }
+            const bool moved = b[0] != pb[0] || b[1] != pb[1] || b[2] != pb[2];
+            flush(moved && k > 0);
+            if (on) {
+                pb[0] = b[0]; pb[1] = b[1]; pb[2] = b[2];
 #pragma unroll
                 for (int c = 0; c < 8; ++c) {
                     const float cw = corner_w(w, c);
@@ -383,8 +459,8 @@ __global__ void __launch_bounds__(128, 4) scatter_kernel(const __grid_constant__
                     for (int v = 0; v < NV; ++v) s[c][v] = fmaf(cw, val[v], s[c][v]);
                 }
             }
-            flush();
         }
+        flush(n > 0);
     }
 }
 
@@ -434,26 +510,34 @@ inline RecLayout record_layout(int L, bool dist, int64_t n_rays) {
     return a;
 }
 
-// Scratch of the passes on the density channel: its plane, then the pixel-tile order of
-// the rays (n_rays = 0: the plane alone).
+// Scratch of the passes on the density channel: its plane, with `grad` a plane of its
+// gradient, then the pixel-tile order of the rays (n_rays = 0: none).
 struct PlaneLayout {
-    size_t plane, bins, perm, bytes;
+    size_t counter, plane, grad, bins, perm, bytes;
 };
 
-inline PlaneLayout plane_layout(int64_t entries, int64_t n_rays) {
+inline PlaneLayout plane_layout(int64_t entries, int64_t n_rays, bool grad = false) {
     PlaneLayout a;
     auto up = [](size_t v) { return (v + 255) / 256 * 256; };
-    a.plane = 0;
-    a.bins = up((size_t)entries * sizeof(float));
+    a.counter = 0;  // tiles handed out at run time
+    a.plane = 256;
+    a.grad = a.plane + up((size_t)entries * sizeof(float));
+    a.bins = a.grad + (grad ? up((size_t)entries * sizeof(float)) : 0);
     const bool order = n_rays >= kRecordMinRays && n_rays <= 0x7FFFFFFF;
     a.perm = a.bins + (order ? (size_t)kMaxBins * sizeof(uint32_t) : 0);
     a.bytes = a.perm + (order ? up((size_t)n_rays * sizeof(int32_t)) : 0) + 256;
     return a;
 }
 
-// Fills the plane (backward.cu) and, with order, the rays' order into p; scratch of
+// Fills the plane (backward.cu) and, with order, the rays' order and the tile counter into
+// p; scratch of
 // plane_layout(entries, order ? p.n_rays : 0).
 void density_scratch(MarchParams& p, int64_t entries, bool order, void* scratch, cudaStream_t st);
+
+// The gradient plane of plane_layout(entries, 0, true), zeroed; and its values added to
+// channel 0 of the table gradient.
+float* gradient_plane(int64_t entries, void* scratch, cudaStream_t st);
+void add_gradient_plane(const float* plane, int64_t entries, float* g_tables, cudaStream_t st);
 
 // The Eq. 8 scenes on FP32 tables with at least this many rows (a level stack that L1 and
 // L2 hold whole gains nothing from a copy): the passes on the density channel take its
@@ -474,15 +558,6 @@ inline size_t record_scratch_bytes(int L, bool dist, int64_t n_rays) {
 // order, or NULL where the rays stay in the given order.
 const int32_t* bin_rays(const MarchParams& m, uint32_t* bins, int32_t* perm, cudaStream_t st);
 
-template <class Kernel>
-unsigned resident_grid(Kernel k, int* cache) {
-    int dev = 0;
-    cudaGetDevice(&dev);
-    if (dev < 0 || dev >= 16) dev = 0;
-    if (!cache[dev]) cache[dev] = resident_blocks(k, 0);
-    return (unsigned)cache[dev];
-}
-
 // Records and scatter of all rays of p.m; rest(p) finishes the rays of p.list.
 template <int L, bool kDist, class Rest>
 void launch_records(RecParams p, void* scratch, cudaStream_t st, Rest rest) {
@@ -498,15 +573,18 @@ void launch_records(RecParams p, void* scratch, cudaStream_t st, Rest rest) {
     p.rec = reinterpret_cast<float*>(base + a.rec);
     p.max_chunks = a.max_chunks;
     p.perm = bin_rays(p.m, reinterpret_cast<uint32_t*>(base + a.bins), reinterpret_cast<int32_t*>(base + a.perm), st);
-    static int cache1[16] = {0}, cache2[16] = {0};
-    const unsigned g1 = resident_grid(record_kernel<L, kDist>, cache1), g2 = resident_grid(scatter_kernel<L, kDist>, cache2);
+    static int cache1[16] = {0}, cache2[16] = {0}, cache3[16] = {0};
+    const unsigned g1 = resident_grid(record_kernel<L, kDist>, cache1),
+                   g2 = resident_grid(scatter_levels_kernel<L, kDist>, cache2),
+                   g3 = resident_grid(scatter_logits_kernel<L, kDist>, cache3);
     for (int64_t r0 = 0; r0 < n; r0 += kRecordRays) {
         p.ray0 = r0;
         p.n_rays = n - r0 < kRecordRays ? n - r0 : kRecordRays;
         cudaMemsetAsync(base + a.counters, 0, 256, st);
         const unsigned blocks = (unsigned)((p.n_rays + 127) / 128);
         record_kernel<L, kDist><<<blocks < g1 ? blocks : g1, 128, 0, st>>>(p);
-        scatter_kernel<L, kDist><<<g2, 128, 0, st>>>(p);
+        scatter_levels_kernel<L, kDist><<<g2, 128, 0, st>>>(p);
+        if (p.m.opts.attn_mode != 1) scatter_logits_kernel<L, kDist><<<g3, 128, 0, st>>>(p);
         rest(p, blocks);
     }
 }
