@@ -161,17 +161,49 @@ __device__ __forceinline__ float2 ffma2(float2 a, float2 b, float2 c) {
 constexpr int kLevelUnroll = NGPRT_LEVEL_UNROLL;
 constexpr int kScatterUnroll = NGPRT_SCATTER_UNROLL;
 
-// Where the gates of Eq. 8 come from.  FP32 and BF16 tables: each level interpolates its
-// own two logits when its turn comes (8 loads of one pair).  The 2L sums are then not
-// all held at once, nothing passes through shared memory (which is carved out of L1),
-// and the level loop has the registers that the 40 coarse channels took: hd 1080p FP32
-// 12.52 -> 11.52 ms with the blocks below, BF16 (1283 x 721) 7.2 -> 5.0 ms (it spilled
-// 460 B a thread).  FP16 tables keep the coarse rows in one pass with the gates in
-// shared memory: half2 sums need half the registers, and the extra loads cost more
-// than they free (6.77 ms against 7.51).
-template <int DT, int AGG>
+// Where the gates of Eq. 8 come from.  The logits of gate_group() levels at a time are
+// interpolated when the first of those levels comes (one load per corner and group), and
+// the gates handed from level to level in registers: the 2L sums are not all held at
+// once, and nothing passes through shared memory, which is carved out of the L1 that the
+// gathers live on.  hd scene: BF16 tables (1283 x 721) 4.69 ms with groups of 4, 4.76 with
+// 2, 4.99 one by one, 7.24 with all logits up front (460 bytes of spills); FP16 1080p 6.56,
+// 6.81, 7.38 and 6.66; FP32 1080p 11.57, 11.63, 11.41 and 12.5, and one by one it is.
+// FP16 stacks of 1, 2 or 3 levels keep all logits up front, with the gates in shared memory:
+// their rows are too narrow for wide loads of a group (paper shape, L = 2: 3.25 ms
+// against 3.47).
+template <int L, int DT, int AGG>
 constexpr bool fly_gates() {
-    return AGG == NGPRT_AGG_SEPARATE_V && DT != NGPRT_F16;
+    return AGG == NGPRT_AGG_SEPARATE_V && (DT != NGPRT_F16 || L % 4 == 0);
+}
+template <int L, int DT>
+constexpr int gate_group() {
+    return DT == NGPRT_F32 || L % 2 != 0 ? 1 : L % 4 == 0 ? 4 : 2;
+}
+
+// G consecutive 32-bit words (aligned to all of them).
+template <int G>
+__device__ __forceinline__ void load_words(const void* p, uint32_t x[G]) {
+    if constexpr (G == 4) {
+        const uint4 q = __ldg(static_cast<const uint4*>(p));
+        x[0] = q.x; x[1] = q.y; x[2] = q.z; x[3] = q.w;
+    } else if constexpr (G == 2) {
+        const uint2 q = __ldg(static_cast<const uint2*>(p));
+        x[0] = q.x; x[1] = q.y;
+    } else {
+        x[0] = __ldg(static_cast<const uint32_t*>(p));
+    }
+}
+
+// The first NF 16-bit channels of a coarse row of NC, as pairs.
+template <int NC, int NF>
+__device__ __forceinline__ void load_row_pairs(const uint16_t* row, uint32_t q[NF / 2]) {
+    if constexpr (NF == NC) load_pairs<NC>(row, q);
+    else {
+        static_assert(NF == kNFeat, "the feature channels");
+        constexpr int G = NC % 8 == 0 ? 4 : NC % 4 == 0 ? 2 : 1;
+#pragma unroll
+        for (int k = 0; k < NF / 2; k += G) load_words<G>(row + 2 * k, q + k);
+    }
 }
 
 // The first NF of a coarse row's NC channels, FP32 or BF16 (NF = 8: the loads that the
@@ -211,30 +243,71 @@ __device__ __forceinline__ void load_row_channels(const void* base, uint32_t ver
     }
 }
 
-// Gates omega^l, beta^l of one level from its two logits at the 8 coarse corners.
-template <int DT, int NC>
+// Gates omega, beta of levels l .. l + G - 1 (FP32 and BF16 grids).
+template <int DT, int NC, int G>
 __device__ __forceinline__ void level_gates(const Grid& g, uint32_t cb, uint32_t sy, uint32_t sz, const float w[3],
-                                            int l, int attn_mode, float& om, float& be) {
+                                            int l, int attn_mode, float om[G], float be[G]) {
     if (attn_mode == 1) {
-        om = be = 1.0f;
+#pragma unroll
+        for (int j = 0; j < G; ++j) om[j] = be[j] = 1.0f;
         return;
     }
-    float2 lg = make_float2(0.0f, 0.0f);
+    float2 lg[G];
+#pragma unroll
+    for (int j = 0; j < G; ++j) lg[j] = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int c = 0; c < 8; ++c) {
         const uint32_t v = cb + (uint32_t)(c & 1) + sy * (uint32_t)((c >> 1) & 1) + sz * (uint32_t)((c >> 2) & 1);
         const float cw = corner_w(w, c);
-        float2 q;
+        const size_t at = (size_t)v * NC + kNFeat + 2 * l;
+        float q[2 * G];
         if constexpr (DT == NGPRT_F32) {
-            q = __ldg(reinterpret_cast<const float2*>(static_cast<const float*>(g.coarse) + (size_t)v * NC + kNFeat) + l);
+            const float* p = static_cast<const float*>(g.coarse) + at;
+            if constexpr (G == 4) load_entry<NGPRT_F32>(p, 0, q);
+            else if constexpr (G == 2) {
+                const float4 x = __ldg(reinterpret_cast<const float4*>(p));
+                q[0] = x.x; q[1] = x.y; q[2] = x.z; q[3] = x.w;
+            } else {
+                const float2 x = __ldg(reinterpret_cast<const float2*>(p));
+                q[0] = x.x; q[1] = x.y;
+            }
         } else {
-            const uint32_t x = __ldg(reinterpret_cast<const uint32_t*>(static_cast<const uint16_t*>(g.coarse) + (size_t)v * NC + kNFeat) + l);
-            q = make_float2(__uint_as_float(x << 16), __uint_as_float(x & 0xFFFF0000u));
+            uint32_t x[G];
+            load_words<G>(static_cast<const uint16_t*>(g.coarse) + at, x);
+#pragma unroll
+            for (int j = 0; j < G; ++j) {
+                q[2 * j] = __uint_as_float(x[j] << 16);
+                q[2 * j + 1] = __uint_as_float(x[j] & 0xFFFF0000u);
+            }
         }
-        lg = ffma2(make_float2(cw, cw), q, lg);
+#pragma unroll
+        for (int j = 0; j < G; ++j) lg[j] = ffma2(make_float2(cw, cw), make_float2(q[2 * j], q[2 * j + 1]), lg[j]);
     }
-    om = gate_sigmoid(lg.x);
-    be = attn_mode == 2 ? om : gate_sigmoid(lg.y);
+#pragma unroll
+    for (int j = 0; j < G; ++j) {
+        om[j] = gate_sigmoid(lg[j].x);
+        be[j] = attn_mode == 2 ? om[j] : gate_sigmoid(lg[j].y);
+    }
+}
+
+// The same for FP16 grids, in packed half2 sums, as pairs.
+template <int NC, int G>
+__device__ __forceinline__ void level_gates_h2(const Grid& g, uint32_t cb, uint32_t sy, uint32_t sz,
+                                               const __half2 cw[4], int l, int attn_mode, __half2 gp[G]) {
+#pragma unroll
+    for (int j = 0; j < G; ++j) gp[j] = __float2half2_rn(attn_mode == 1 ? 1.0f : 0.0f);
+    if (attn_mode == 1) return;
+#pragma unroll
+    for (int c = 0; c < 8; ++c) {
+        const uint32_t v = cb + (uint32_t)(c & 1) + sy * (uint32_t)((c >> 1) & 1) + sz * (uint32_t)((c >> 2) & 1);
+        uint32_t x[G];
+        load_words<G>(static_cast<const uint16_t*>(g.coarse) + (size_t)v * NC + kNFeat + 2 * l, x);
+        const __half2 cw2 = corner_h2(cw, c);
+#pragma unroll
+        for (int j = 0; j < G; ++j) gp[j] = __hfma2(cw2, *reinterpret_cast<const __half2*>(&x[j]), gp[j]);
+    }
+#pragma unroll
+    for (int j = 0; j < G; ++j) gp[j] = gate_sigmoid_h2(attn_mode == 2 ? __low2half2(gp[j]) : gp[j]);
 }
 
 // Eq. 6-8 at unit-cube position u: f = f~ + Att(f^1..f^L; a), or one of the
@@ -253,7 +326,8 @@ __device__ __forceinline__ void level_gates(const Grid& g, uint32_t cb, uint32_t
 // f^l in the slots [8l, 8l + 8) and its 64 hidden pre-activations in [8L, 8L + 64).
 // With kRec (the reverse pass's records, Eq. 8), gates is the record's level fields and
 // every level leaves omega^l, beta^l, sigma^l and q^l in its four.
-template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V, bool kKeep = false, bool kRec = false>
+template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V, bool kKeep = false, bool kRec = false,
+          int G = gate_group<L, DT>()>
 __device__ __forceinline__ void sample_features(const Grid& g, const float u[3], int attn_mode, float f[8],
                                                 float* gates, int stride, const float* gq = nullptr) {
     constexpr int NC = coarse_channels(L, AGG);
@@ -263,8 +337,11 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
     // level) and each level's gated sum is taken in mixed precision (FP16 factors,
     // FP32 sum), without converting the level's features
     constexpr bool kHalfGates = DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V && !kKeep;
-    constexpr bool kFly = fly_gates<DT, AGG>() && !kKeep;
+    constexpr bool kFly = fly_gates<L, DT, AGG>() && !kKeep;
     constexpr int NF = kFly ? kNFeat : NC;  // channels taken from the coarse rows up front
+    // the gates of the levels to come, the next level's first
+    [[maybe_unused]] float og[G], bg[G];
+    [[maybe_unused]] __half2 hg[G], ccw[4];
     uint32_t ufx[3] = {0u, 0u, 0u};
     if constexpr (DT != NGPRT_F32) {
 #pragma unroll
@@ -279,23 +356,24 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
     coarse_base(g, b, cb, sy, sz);
     if constexpr (DT == NGPRT_F16) {
         // FP16 tables: trilinear sums in packed half2 FMAs, converted once
-        __half2 hacc[NC / 2], cw[4];
+        __half2 hacc[NF / 2];
+        __half2(&cw)[4] = ccw;
         corner_w_h2(w, cw);
 #pragma unroll
-        for (int ch = 0; ch < NC / 2; ++ch) hacc[ch] = __float2half2_rn(0.0f);
+        for (int ch = 0; ch < NF / 2; ++ch) hacc[ch] = __float2half2_rn(0.0f);
 #pragma unroll
         for (int c = 0; c < 8; ++c) {
             const uint32_t v = cb + (uint32_t)(c & 1) + sy * (uint32_t)((c >> 1) & 1) + sz * (uint32_t)((c >> 2) & 1);
-            uint32_t q[NC / 2];
-            load_pairs<NC>(static_cast<const uint16_t*>(g.coarse) + (size_t)v * NC, q);
+            uint32_t q[NF / 2];
+            load_row_pairs<NC, NF>(static_cast<const uint16_t*>(g.coarse) + (size_t)v * NC, q);
             const __half2 cw2 = corner_h2(cw, c);
 #pragma unroll
-            for (int ch = 0; ch < NC / 2; ++ch)
+            for (int ch = 0; ch < NF / 2; ++ch)
                 hacc[ch] = __hfma2(cw2, *reinterpret_cast<const __half2*>(&q[ch]), hacc[ch]);
         }
 #pragma unroll
-        for (int ch = 0; ch < (kHalfGates ? kNFeat / 2 : NC / 2); ++ch) acc[ch] = __half22float2(hacc[ch]);
-        if constexpr (kHalfGates) {
+        for (int ch = 0; ch < (kHalfGates ? kNFeat / 2 : NF / 2); ++ch) acc[ch] = __half22float2(hacc[ch]);
+        if constexpr (kHalfGates && !kFly) {
 #pragma unroll
             for (int l = 0; l < L; ++l) {
                 const __half2 lg = hacc[kNFeat / 2 + l];
@@ -391,7 +469,15 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
                 for (int ch = 0; ch < 4; ++ch) h[ch] = __hfma2(cw2, e2[ch], h[ch]);
             }
             if constexpr (kHalfGates) {
-                const __half2 gp = reinterpret_cast<const __half2*>(gates)[l * stride];
+                __half2 gp;
+                if constexpr (kFly) {
+                    if (G == 1 || l % G == 0) level_gates_h2<NC, G>(g, cb, sy, sz, ccw, l, attn_mode, hg);
+                    gp = hg[0];
+#pragma unroll
+                    for (int j = 0; j + 1 < G; ++j) hg[j] = hg[j + 1];
+                } else {
+                    gp = reinterpret_cast<const __half2*>(gates)[l * stride];
+                }
                 const __half om = __low2half(gp), be = __high2half(gp);
                 f[0] = fma_f16_f32(om, __low2half(h[0]), f[0]);
                 f[1] = fma_f16_f32(be, __high2half(h[0]), f[1]);
@@ -478,8 +564,16 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
         } else if constexpr (!kHalfGates) {
             // packed pairs: each half is the scalar fmaf, bit for bit
             float om, be;
-            if constexpr (kFly) level_gates<DT, NC>(g, cb, sy, sz, w, l, attn_mode, om, be);
-            else {
+            if constexpr (kFly) {
+                if (G == 1 || l % G == 0) level_gates<DT, NC, G>(g, cb, sy, sz, w, l, attn_mode, og, bg);
+                om = og[0];
+                be = bg[0];
+#pragma unroll
+                for (int j = 0; j + 1 < G; ++j) {
+                    og[j] = og[j + 1];
+                    bg[j] = bg[j + 1];
+                }
+            } else {
                 om = gates[(2 * l) * stride];
                 be = gates[(2 * l + 1) * stride];
             }
@@ -554,7 +648,8 @@ __device__ __forceinline__ float sample_density(const Grid& g, const float* __re
     for (int a = 0; a < 3; ++a) grid_cell(u[a], g.R_C, b[a], w[a]);
     uint32_t cb, sy, sz;
     coarse_base(g, b, cb, sy, sz);
-    float ccw[8];
+    constexpr int G = L % 4 == 0 ? 4 : 1;  // levels whose gates are interpolated at a time
+    float ccw[8], og[G];
     const float* row[8];
     float f0 = 0.0f;
 #pragma unroll
@@ -576,13 +671,28 @@ __device__ __forceinline__ float sample_density(const Grid& g, const float* __re
         for (int c = 0; c < 8; ++c)
             q[c] = __ldg(tl + level_index_k<kKind>(g, l, (uint32_t)(bl[0] + (c & 1)), (uint32_t)(bl[1] + ((c >> 1) & 1)),
                                                    (uint32_t)(bl[2] + ((c >> 2) & 1))));
-        float om = 1.0f;
-        if (attn_mode != 1) {
-            float lg = 0.0f;
+        if (G == 1 || l % G == 0) {
+            float lg[G];
 #pragma unroll
-            for (int c = 0; c < 8; ++c) lg = fmaf(ccw[c], __ldg(row[c] + kNFeat + 2 * l), lg);
-            om = gate_sigmoid(lg);
+            for (int k = 0; k < G; ++k) lg[k] = 0.0f;
+            if (attn_mode != 1) {
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    // one 32-byte load of four levels' pairs: its beta half is idle, but
+                    // eight instructions a level in place of sixteen are what counts here
+                    float x[2 * G];
+                    if constexpr (G == 4) load_entry<NGPRT_F32>(row[c] + kNFeat + 2 * l, 0, x);
+                    else x[0] = __ldg(row[c] + kNFeat + 2 * l);
+#pragma unroll
+                    for (int k = 0; k < G; ++k) lg[k] = fmaf(ccw[c], x[2 * k], lg[k]);
+                }
+            }
+#pragma unroll
+            for (int k = 0; k < G; ++k) og[k] = attn_mode == 1 ? 1.0f : gate_sigmoid(lg[k]);
         }
+        const float om = og[0];
+#pragma unroll
+        for (int k = 0; k + 1 < G; ++k) og[k] = og[k + 1];
         float sg = 0.0f;
 #pragma unroll
         for (int c = 0; c < 8; ++c) sg = fmaf(corner_w(wl, c), q[c], sg);
@@ -605,12 +715,10 @@ __device__ __forceinline__ float sample_density(const Grid& g, const float* __re
     return f0;
 }
 
-// Shared-memory floats per thread that sample_features parks its gates in (forward
-// form).  What shared memory takes is lost to L1, which holds the coarse rows and the
-// dense levels.
+// Shared-memory floats per thread that sample_features parks its gates in.
 template <int L, int DT, int AGG>
 __host__ __device__ constexpr int gate_floats() {
-    if (AGG == NGPRT_AGG_SUM || AGG == NGPRT_AGG_MLP || fly_gates<DT, AGG>()) return 0;
+    if (AGG == NGPRT_AGG_SUM || AGG == NGPRT_AGG_MLP || fly_gates<L, DT, AGG>()) return 0;
     return DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V ? L : 2 * L;
 }
 
@@ -941,17 +1049,18 @@ __device__ __forceinline__ bool ray_setup(const MarchParams& p, int64_t& ray, Ra
 // hd scene, 1080p: FP16 9.46 -> 8.98 ms, FP32 16.05 -> 15.60 ms).
 // Blocks per SM the register allocation must allow (hd scene, L = 16): FP32 tables with 4
 // or more levels 7 (72 registers; 1080p 11.5 ms against 12.0 at 5, 11.7 at 6 and 12.0 at
-// 8), FP16 tables 8 (64 registers; 6.77 ms against 6.83 at 7), BF16 tables 8 (5.00 ms
-// against 5.12 at 7 and 5.23 at 10); FP32 with fewer levels 8.  The other aggregation
-// forms of FP32 and BF16 tables hold more and keep 5 and 7; the MLP form keeps its 64
-// hidden units in registers.
+// 8), FP16 tables 8 (64 registers; 6.55 ms against 6.68 at 7 and 6.63 at 9), BF16 tables 7
+// (4.65 ms against 4.75 at 6 and 4.68 at 8); FP32 with fewer levels 8.  The other
+// aggregation forms of FP32 and BF16 tables hold more and keep 5 and 7; the MLP form keeps
+// its 64 hidden units in registers.
 template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V>
 constexpr int march_min_blocks() {
     if (AGG == NGPRT_AGG_MLP) return 3;
     if (NGPRT_MARCH_MIN_BLOCKS > 0) return NGPRT_MARCH_MIN_BLOCKS;
     if (DT == NGPRT_F16) return 8;
-    if (AGG != NGPRT_AGG_SEPARATE_V) return DT == NGPRT_BF16 ? 7 : L >= 4 ? 5 : 8;
-    return DT == NGPRT_F32 && L >= 4 ? 7 : 8;
+    if (DT == NGPRT_BF16) return 7;
+    if (AGG != NGPRT_AGG_SEPARATE_V) return L >= 4 ? 5 : 8;
+    return L >= 4 ? 7 : 8;
 }
 
 template <int L, int DT, int AGG>
@@ -1012,6 +1121,7 @@ template <int L, int DT, int AGG>
 __global__ void __launch_bounds__(128, 3)
     march_group_kernel(const __grid_constant__ MarchParams p, int g_log2) {
     extern __shared__ float gate_smem[];
+    constexpr int GG = L % 4 == 0 ? 4 : L % 2 == 0 ? 2 : 1;
     const int G = 1 << g_log2;
     const int64_t rl = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> g_log2;
     const int lig = threadIdx.x & (G - 1);
@@ -1043,7 +1153,10 @@ __global__ void __launch_bounds__(128, 3)
             }
             float f[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, trans = 1.0f;
             if (lig < n) {
-                sample_features<L, DT, AGG>(p.g, my_u, p.opts.attn_mode, f, gate_smem + threadIdx.x, blockDim.x);
+                // what it waits on is the chain of loads: the widest groups of gates (50001
+                // rays, forward and reverse pass: 2190 us against 2263 one by one)
+                sample_features<L, DT, AGG, false, false, GG>(p.g, my_u, p.opts.attn_mode, f, gate_smem + threadIdx.x,
+                                                              blockDim.x);
                 trans = expf(-expf(f[0]) * my_delta);
             }
             __syncwarp(mask);
