@@ -132,7 +132,7 @@ __global__ void __launch_bounds__(128) distortion_backward_kernel(const __grid_c
 // set), or NULL.
 template <int L>
 void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, float* g_plane, cudaStream_t st) {
-    const size_t shm = (size_t)2 * L * 128 * sizeof(float);
+    const size_t shm = (size_t)gate_floats<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V>() * 128 * sizeof(float);
     if (!backward) {
         if (p.m.plane) {
             static int cache[16] = {0};
@@ -244,7 +244,7 @@ static int32_t run_distortion(bool backward, const ngprt_scene* scene, const ngp
     }
     void* records = nullptr;
     float* g_plane = nullptr;
-    if (workspace && plane_serves(scene)) {
+    if (workspace && plane_serves(scene) && !lattice(p.m)) {
         const int64_t entries = ngprt_table_entries(scene);
         const size_t plane = plane_layout(entries, backward ? 0 : n_rays, backward).bytes;
         const size_t rec = backward ? record_scratch_bytes(L, true, n_rays) : 0;

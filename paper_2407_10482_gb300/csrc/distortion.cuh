@@ -27,13 +27,15 @@ struct DistSampler {
         const float m = fmaf(0.5f, delta, t);
         Lp = fmaf(2.0f * w, fmaf(m, W, -S), Lp);
         Ls = fmaf(w * w, delta * (1.0f / 3.0f), Ls);
-        W += w;
+        // rounded by itself, as in the reverse pass: that pass subtracts running sums from
+        // these totals
+        W = fadd(W, w);
         S = fmaf(w, m, S);
         return stop;
     }
 };
 
-template <class Weights>
+template <bool kSnap, class Weights>
 __device__ __forceinline__ void distortion_ray(const DistParams& p, const Weights& weights, int64_t tile = -1) {
     int64_t ray = 0;
     Ray ry;
@@ -43,7 +45,7 @@ __device__ __forceinline__ void distortion_ray(const DistParams& p, const Weight
     if (has_ray) {
         DistSampler<Weights> smp{weights, 0.0f, 0.0f, 0.0f, 0.0f};
         int n_march = 0, n_samp = 0;
-        if (hit) march_loop(p.m, ry, smp, n_march, n_samp);
+        if (hit) march_loop<kSnap>(p.m, ry, smp, n_march, n_samp);
         Ld = smp.Lp + smp.Ls;
         reinterpret_cast<float4*>(p.dist_state)[ray] = make_float4(Ld, smp.W, smp.S, 0.0f);
     }
@@ -59,7 +61,7 @@ __device__ __forceinline__ void distortion_ray(const DistParams& p, const Weight
 template <int L, int AGG>
 __global__ void __launch_bounds__(128) distortion_kernel(const __grid_constant__ DistParams p) {
     extern __shared__ float gate_smem[];
-    distortion_ray(p, ForwardSampler<L, NGPRT_F32, AGG>(p.m.g, p.m.opts.attn_mode, p.m.opts.t_term,
+    distortion_ray<true>(p, ForwardSampler<L, NGPRT_F32, AGG>(p.m.g, p.m.opts.attn_mode, p.m.opts.t_term,
                                                         gate_smem + threadIdx.x));
 }
 
@@ -67,7 +69,7 @@ __global__ void __launch_bounds__(128) distortion_kernel(const __grid_constant__
 template <int L>
 __global__ void __launch_bounds__(128, kWeightMinBlocks) distortion_plane_kernel(const __grid_constant__ DistParams p) {
     for (int64_t tile; (tile = next_tile(p.m)) >= 0;) {
-        distortion_ray(p, WeightSampler<L>(p.m.g, p.m.plane, p.m.opts.attn_mode, p.m.opts.t_term), tile);
+        distortion_ray<false>(p, WeightSampler<L>(p.m.g, p.m.plane, p.m.opts.attn_mode, p.m.opts.t_term), tile);
         __syncwarp();
     }
 }

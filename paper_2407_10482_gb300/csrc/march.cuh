@@ -168,12 +168,15 @@ constexpr int kScatterUnroll = NGPRT_SCATTER_UNROLL;
 // gathers live on.  hd scene: BF16 tables (1283 x 721) 4.69 ms with groups of 4, 4.76 with
 // 2, 4.99 one by one, 7.24 with all logits up front (460 bytes of spills); FP16 1080p 6.56,
 // 6.81, 7.38 and 6.66; FP32 1080p 11.57, 11.63, 11.41 and 12.5, and one by one it is.
-// FP16 stacks of 1, 2 or 3 levels keep all logits up front, with the gates in shared memory:
-// their rows are too narrow for wide loads of a group (paper shape, L = 2: 3.25 ms
-// against 3.47).
+// Stacks of 1, 2 or 3 levels keep all logits up front, with the gates in shared memory: there
+// are few of them, and their rows are too narrow for wide loads of a group (paper shape,
+// L = 2: FP16 3.25 ms against 3.47, FP32 4.71 against 5.12; BF16 3.74 against 9.73, where
+// the warp's lanes no longer sampled together).  So do FP32 tables of up to 8 levels (1283 x
+// 721: L = 4 617 us against 706, L = 8 3.03 ms against 3.15).
 template <int L, int DT, int AGG>
 constexpr bool fly_gates() {
-    return AGG == NGPRT_AGG_SEPARATE_V && (DT != NGPRT_F16 || L % 4 == 0);
+    if (AGG != NGPRT_AGG_SEPARATE_V || L < 4) return false;
+    return DT == NGPRT_F32 ? L > 8 : DT == NGPRT_BF16 || L % 4 == 0;
 }
 template <int L, int DT>
 constexpr int gate_group() {
@@ -337,7 +340,7 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
     // level) and each level's gated sum is taken in mixed precision (FP16 factors,
     // FP32 sum), without converting the level's features
     constexpr bool kHalfGates = DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V && !kKeep;
-    constexpr bool kFly = fly_gates<L, DT, AGG>() && !kKeep;
+    constexpr bool kFly = (kRec || fly_gates<L, DT, AGG>()) && !kKeep;
     constexpr int NF = kFly ? kNFeat : NC;  // channels taken from the coarse rows up front
     // the gates of the levels to come, the next level's first
     [[maybe_unused]] float og[G], bg[G];
@@ -839,6 +842,9 @@ __device__ __forceinline__ float empty_step(int bounded, const float x[3], const
 // Returns true with u (unit-cube position), delta (clipped sample step) and dt (the
 // sample step) of the point at st.t, or false when the ray is exhausted (t_out or a
 // cap reached).
+// kSnap = false (callers that hold lattice_snap off): the lattice's origin and index need
+// not be kept (paper-shaped L = 2 frame 3.26 -> 3.13 ms, small view 77 -> 74 us).
+template <bool kSnap = true>
 __device__ __forceinline__ bool march_advance(const MarchParams& p, const Ray& ry, MarchState& st, float u[3],
                                               float& delta, float& dt) {
     const ngprt_render_opts& op = p.opts;
@@ -851,7 +857,7 @@ __device__ __forceinline__ bool march_advance(const MarchParams& p, const Ray& r
     // side of a finest voxel, a power of two: a level's is its exact multiple
     const float v0 = fdiv(2.0f * B, (float)R_O);
     const float guard = fmul(kEmptyGuard, v0);
-    const bool snap = op.lattice_snap && bounded;
+    const bool snap = kSnap && op.lattice_snap && bounded;
     while (df_lt(st.t, st.t_out) && st.n_march < op.max_march && st.n_samp < op.max_samples) {
         ++st.n_march;
         float x[3], y[3], r, ir, kc;
@@ -901,9 +907,10 @@ __device__ __forceinline__ bool march_advance(const MarchParams& p, const Ray& r
 }
 
 // Move past the sample just taken at st.t (sample step dt, or the next lattice point).
+template <bool kSnap = true>
 __device__ __forceinline__ void march_after_sample(const MarchParams& p, MarchState& st, float dt) {
     ++st.n_samp;
-    if (p.opts.lattice_snap && p.g.bounded) {
+    if (kSnap && p.opts.lattice_snap && p.g.bounded) {
         st.lat_k += 1;
         st.t = df_add(st.t_start, df_prod((float)st.lat_k, fmul(p.opts.step_base, p.opts.step_gamma)));
     } else {
@@ -915,24 +922,24 @@ __device__ __forceinline__ void march_after_sample(const MarchParams& p, MarchSt
 // marching point and returns true when the ray terminates.  The lanes of a warp
 // first advance through empty space each to its own next sample, then sample
 // together.
-template <class Sampler>
+template <bool kSnap = true, class Sampler>
 __device__ __forceinline__ void march_loop_from(const MarchParams& p, const Ray& ry, MarchState& st, Sampler& smp) {
     float u[3], delta, dt;
-    while (march_advance(p, ry, st, u, delta, dt)) {
+    while (march_advance<kSnap>(p, ry, st, u, delta, dt)) {
         const bool stop = smp.sample(u, df_float(st.t), delta);
         if (stop) {
             ++st.n_samp;
             break;
         }
-        march_after_sample(p, st, dt);
+        march_after_sample<kSnap>(p, st, dt);
     }
 }
 
-template <class Sampler>
+template <bool kSnap = true, class Sampler>
 __device__ __forceinline__ void march_loop(const MarchParams& p, const Ray& ry, Sampler& smp, int& n_march,
                                            int& n_samp) {
     MarchState st = march_state(ry);
-    march_loop_from(p, ry, st, smp);
+    march_loop_from<kSnap>(p, ry, st, smp);
     n_march = st.n_march;
     n_samp = st.n_samp;
 }
@@ -1017,11 +1024,14 @@ struct WeightSampler {
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
         const float sigma = expf(sample_density<L>(g, plane, u, attn_mode));
         const float trans = expf(-sigma * delta);
-        w_last = T * (1.0f - trans);
-        T *= trans;
+        w_last = fmul(T, fsub(1.0f, trans));
+        T = fmul(T, trans);
         return T < t_term;
     }
 };
+
+// Whether the samples stay on a lattice (lattice_snap has no effect on contracted scenes).
+__host__ __device__ __forceinline__ bool lattice(const MarchParams& p) { return p.opts.lattice_snap && p.g.bounded; }
 
 // Ray set-up shared by every pass: this thread's ray and its domain interval
 // (false if the lane has no ray; hit = the interval is not empty).
@@ -1047,10 +1057,11 @@ __device__ __forceinline__ bool ray_setup(const MarchParams& p, int64_t& ray, Ra
 // 32 listed rays) from the counter until none are left: a warp that finishes early
 // starts another tile instead of idling until its block's slowest warp ends (fitted
 // hd scene, 1080p: FP16 9.46 -> 8.98 ms, FP32 16.05 -> 15.60 ms).
-// Blocks per SM the register allocation must allow (hd scene, L = 16): FP32 tables with 4
-// or more levels 7 (72 registers; 1080p 11.5 ms against 12.0 at 5, 11.7 at 6 and 12.0 at
+// Blocks per SM the register allocation must allow (hd scene, L = 16): FP32 tables with more
+// than 8 levels 7 (72 registers; 1080p 11.5 ms against 12.0 at 5, 11.7 at 6 and 12.0 at
 // 8), FP16 tables 8 (64 registers; 6.55 ms against 6.68 at 7 and 6.63 at 9), BF16 tables 7
-// (4.65 ms against 4.75 at 6 and 4.68 at 8); FP32 with fewer levels 8.  The other
+// (4.65 ms against 4.75 at 6 and 4.68 at 8); FP32 of 4 to 8 levels
+// holds all gates and takes 5, of fewer levels 8.  The other
 // aggregation forms of FP32 and BF16 tables hold more and keep 5 and 7; the MLP form keeps
 // its 64 hidden units in registers.
 template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V>
@@ -1060,15 +1071,17 @@ constexpr int march_min_blocks() {
     if (DT == NGPRT_F16) return 8;
     if (DT == NGPRT_BF16) return 7;
     if (AGG != NGPRT_AGG_SEPARATE_V) return L >= 4 ? 5 : 8;
-    return L >= 4 ? 7 : 8;
+    return L > 8 ? 7 : L >= 4 ? 5 : 8;
 }
 
-template <int L, int DT, int AGG>
-__global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
-    march_kernel(const __grid_constant__ MarchParams p) {
+constexpr int kWideBlocks = 5;
+
+// kBlocks: blocks per SM (march_min_blocks, or kWideBlocks for small batches).
+template <int L, int DT, int AGG, int kBlocks>
+__global__ void __launch_bounds__(128, kBlocks) march_kernel(const __grid_constant__ MarchParams p) {
     extern __shared__ float gate_smem[];
     // one ray of this thread (of the warp's tile `tile`, or -1: by the thread index)
-    auto one_ray = [&](int64_t tile) {
+    auto one_ray = [&](int64_t tile, auto snap) {
         int64_t ray;
         Ray ry;
         bool hit;
@@ -1082,7 +1095,7 @@ __global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
         }
         ForwardSampler<L, DT, AGG> smp(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x);
         int n_march = 0, n_samp = 0;
-        if (hit) march_loop(p, ry, smp, n_march, n_samp);
+        if (hit) march_loop<decltype(snap)::value>(p, ry, smp, n_march, n_samp);
         reinterpret_cast<float4*>(s)[0] = make_float4(smp.Cd[0], smp.Cd[1], smp.Cd[2], smp.F[0]);
         reinterpret_cast<float4*>(s)[1] = make_float4(smp.F[1], smp.F[2], smp.F[3], smp.A);
         reinterpret_cast<float4*>(s)[2] = make_float4(smp.depth, ry.dh[0], ry.dh[1], ry.dh[2]);
@@ -1096,12 +1109,17 @@ __global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
             }
         }
     };
-    if (!p.tile_counter) {
-        one_ray(-1);
+    if (!p.tile_counter || lattice(p)) {
+        int64_t tile = -1;  // without the counter: this warp's own, once
+        do {
+            if (p.tile_counter && (tile = next_tile(p)) < 0) break;
+            one_ray(tile, std::true_type{});
+            __syncwarp();
+        } while (p.tile_counter);
         return;
     }
     for (int64_t tile; (tile = next_tile(p)) >= 0;) {
-        one_ray(tile);
+        one_ray(tile, std::false_type{});
         __syncwarp();
     }
 }
@@ -1141,14 +1159,14 @@ __global__ void __launch_bounds__(128, 3)
             float my_u[3] = {0.0f, 0.0f, 0.0f}, my_t = 0.0f, my_delta = 0.0f;
             while (n < G) {
                 float u[3], delta, dt;
-                if (!march_advance(p, ry, st, u, delta, dt)) break;
+                if (!march_advance<false>(p, ry, st, u, delta, dt)) break;
                 if (lig == n) {
                     my_u[0] = u[0]; my_u[1] = u[1]; my_u[2] = u[2];
                     my_t = df_float(st.t);
                     my_delta = delta;
                     my_march = st.n_march;
                 }
-                march_after_sample(p, st, dt);
+                march_after_sample<false>(p, st, dt);
                 ++n;
             }
             float f[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, trans = 1.0f;
@@ -1210,32 +1228,49 @@ unsigned resident_grid(Kernel k, int* cache) {
 template <int L, int DT, int AGG>
 void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
     const size_t shm = (size_t)gate_floats<L, DT, AGG>() * 128 * sizeof(float);  // attention gates of the block's rays
-    // this instantiation's resident blocks, per device, found once
-    static int cache[16] = {0};
+    // the instantiations' resident blocks, per device, found once
     int dev = 0;
     cudaGetDevice(&dev);
     if (dev < 0 || dev >= 16) dev = 0;
-    if (!cache[dev]) cache[dev] = resident_blocks(march_kernel<L, DT, AGG>, shm);
+    constexpr int kBlocks = march_min_blocks<L, DT, AGG>();
     if constexpr (AGG == NGPRT_AGG_SEPARATE_V) {
+        const int64_t rays = p.mode == 0 ? (int64_t)p.tiles_per_view * p.n_cams * 32 : p.n_rays;
         // Several lanes a ray up to 2.4 times the threads that are resident at once: the
         // lanes of a group share the long chain of a ray's samples, which pays even where
-        // the blocks take a second turn (50001 rays: G = 1 2997 us for forward and reverse
-        // pass, G = 2 at 1.3 to 1.7 turns 2714 to 2637), and stops to when the GPU is full
-        // of rays anyway.
-        const int64_t rays = p.mode == 0 ? (int64_t)p.tiles_per_view * p.n_cams * 32 : p.n_rays;
+        // the blocks take a second turn (hd, 57 k FP32 rays: 1387 us at two lanes, 1787 at
+        // one), and stops to when the GPU is full of rays anyway.  FP16 tables from four
+        // lanes on (57 k rays: 1203 us at two, 983 at one).  Stacks of up to 8 levels have
+        // shorter chains: from four lanes on, up to 1.8 times (8 levels, FP32: 18 k rays
+        // 390 us at four lanes, 575 at two or one; 36 k 760, 735 and 707; 68 k BF16 731 us
+        // at two, 508 at one).
+        constexpr bool kShort = L <= 8;
         static int room_cache[16] = {0};
         if (!room_cache[dev]) room_cache[dev] = resident_blocks(march_group_kernel<L, DT, AGG>, shm);
         const int64_t room = (int64_t)room_cache[dev] * 128;
         int g = 0;
-        while (g < 5 && (rays << (g + 1)) * 5 <= room * 12) ++g;
-        if (g > 0 && !p.fb_a_hat) {
+                while (g < 5 && (rays << (g + 1)) * 5 <= room * (kShort ? 9 : 12)) ++g;
+        if (g > (kShort || DT == NGPRT_F16 ? 1 : 0) && !p.fb_a_hat && !lattice(p)) {
             const unsigned blocks = (unsigned)(((rays << g) + 127) / 128);
             march_group_kernel<L, DT, AGG><<<blocks, 128, shm, st>>>(p, g);
             return;
         }
+        // Batches that do not fill the SMs with kBlocks blocks gain nothing from them, and
+        // lose to the spills that buy them: 5 blocks (96 registers) up to 1.5 times their
+        // resident threads.  hd, 77 k rays: FP32 1807 us against 1924, FP16 1002 against
+        // 1139, BF16 1277 against 1387; 120 k: 2074 and 2065, 1141 and 1211, 1471 and 1472;
+        // 224 k: 2578 and 2558, 1487 and 1495, 1932 and 1866.
+        static int wide_cache[16] = {0};
+        if (!wide_cache[dev]) wide_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kWideBlocks>, shm);
+        if (!p.fb_a_hat && rays * 2 <= (int64_t)wide_cache[dev] * 128 * 3) {
+            if (p.tile_counter && grid.x > (unsigned)wide_cache[dev]) grid.x = (unsigned)wide_cache[dev];
+            march_kernel<L, DT, AGG, kWideBlocks><<<grid, 128, shm, st>>>(p);
+            return;
+        }
     }
+    static int cache[16] = {0};
+    if (!cache[dev]) cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kBlocks>, shm);
     if (p.tile_counter && grid.x > (unsigned)cache[dev]) grid.x = (unsigned)cache[dev];
-    march_kernel<L, DT, AGG><<<grid, 128, shm, st>>>(p);
+    march_kernel<L, DT, AGG, kBlocks><<<grid, 128, shm, st>>>(p);
 }
 
 template <int L, int AGG>

@@ -127,7 +127,8 @@ extern "C" int32_t ngprt_occupancy_visibility_ws(const ngprt_scene* scene, const
         return cuda_status(fn);
     }
     const bool built = scene->L <= 4 || scene->L == 8 || scene->L == 16;
-    if (built && workspace && plane_serves(scene) && ws_bytes >= ngprt_density_scratch_bytes(scene, n_rays))
+    if (built && workspace && plane_serves(scene) && !lattice(p) &&
+        ws_bytes >= ngprt_density_scratch_bytes(scene, n_rays))
         density_scratch(p, ngprt_table_entries(scene), true, workspace, st);
     switch (scene->L) {
         case 1: launch_visibility<1, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, grid, w_thr, R, vis, st); break;

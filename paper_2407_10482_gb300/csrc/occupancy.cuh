@@ -73,6 +73,8 @@ __global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
 // The same marks from the density channel alone (p.plane).  Bound by instruction issue
 // (0.71 of one a scheduler and cycle, ALU pipe 56%); tiles handed out at run time, as the
 // render's, were 5% slower here (hd, 4 views of 960 x 540: 7.95 against 7.60 ms).
+// The march keeps the lattice's state here: without it the compiler lets the lanes of a
+// warp sample apart (17.4 ms).
 template <int L>
 __global__ void __launch_bounds__(128, kWeightMinBlocks)
     visibility_plane_kernel(const __grid_constant__ MarchParams p, float w_thr, int32_t R, uint8_t* vis) {
@@ -96,10 +98,11 @@ void launch_density(int dt, const DensityOccParams& p, cudaStream_t st) {
             return;
         }
     }
-    const size_t shm = (size_t)2 * L * 128 * sizeof(float);
-    if (dt == NGPRT_F32) density_occ_kernel<L, NGPRT_F32, AGG><<<blocks, 128, shm, st>>>(p);
-    else if (dt == NGPRT_F16) density_occ_kernel<L, NGPRT_F16, AGG><<<blocks, 128, shm, st>>>(p);
-    else density_occ_kernel<L, NGPRT_BF16, AGG><<<blocks, 128, shm, st>>>(p);
+    const size_t shm = 128 * sizeof(float), f32 = gate_floats<L, NGPRT_F32, AGG>() * shm,
+                 f16 = gate_floats<L, NGPRT_F16, AGG>() * shm, bf16 = gate_floats<L, NGPRT_BF16, AGG>() * shm;
+    if (dt == NGPRT_F32) density_occ_kernel<L, NGPRT_F32, AGG><<<blocks, 128, f32, st>>>(p);
+    else if (dt == NGPRT_F16) density_occ_kernel<L, NGPRT_F16, AGG><<<blocks, 128, f16, st>>>(p);
+    else density_occ_kernel<L, NGPRT_BF16, AGG><<<blocks, 128, bf16, st>>>(p);
 }
 
 template <int L, int AGG>
@@ -111,10 +114,11 @@ void launch_visibility(int dt, const MarchParams& p, dim3 grid, float w_thr, int
             return;
         }
     }
-    const size_t shm = (size_t)2 * L * 128 * sizeof(float);
-    if (dt == NGPRT_F32) visibility_kernel<L, NGPRT_F32, AGG><<<grid, 128, shm, st>>>(p, w_thr, R, vis);
-    else if (dt == NGPRT_F16) visibility_kernel<L, NGPRT_F16, AGG><<<grid, 128, shm, st>>>(p, w_thr, R, vis);
-    else visibility_kernel<L, NGPRT_BF16, AGG><<<grid, 128, shm, st>>>(p, w_thr, R, vis);
+    const size_t shm = 128 * sizeof(float), f32 = gate_floats<L, NGPRT_F32, AGG>() * shm,
+                 f16 = gate_floats<L, NGPRT_F16, AGG>() * shm, bf16 = gate_floats<L, NGPRT_BF16, AGG>() * shm;
+    if (dt == NGPRT_F32) visibility_kernel<L, NGPRT_F32, AGG><<<grid, 128, f32, st>>>(p, w_thr, R, vis);
+    else if (dt == NGPRT_F16) visibility_kernel<L, NGPRT_F16, AGG><<<grid, 128, f16, st>>>(p, w_thr, R, vis);
+    else visibility_kernel<L, NGPRT_BF16, AGG><<<grid, 128, bf16, st>>>(p, w_thr, R, vis);
 }
 
 // The forms of Table 3 other than Eq. 8 (occupancy_agg.cu): L = 2, 4, 16.

@@ -26,6 +26,7 @@
 // job being a level, the coarse feature channels or a group of coarse logits; job-major,
 // so that one level's gradient rows (16.7 MB for a hashed hd level) stay in L2 while all
 // chunks add to them.
+// Marches on a lattice (lattice_snap) keep the one-kernel forms.
 // Rays whose records find no chunk left go to a list (with their first unrecorded
 // sample) that the one-kernel form finishes.
 //
@@ -35,7 +36,7 @@
 // the lanes in pairs; levels and logits in kernels of their own, each with the blocks its
 // registers allow, gave the rest.  The march is bound by the same 180 G sectors a second
 // that its gathers take from L2.  The regulariser at the same rays: 1.9 + 2.8 ms in place
-// of 29.3 (3.6 for the scatter before it had a gradient plane).
+// of 29.3.
 #pragma once
 #include <string.h>
 
@@ -123,7 +124,7 @@ __global__ void __launch_bounds__(128, kDist ? 6 : 4) record_kernel(const __grid
         int slot = kSlots;
         for (;;) {
             float u[3], delta, dt;
-            if (live) live = march_advance(p.m, ry, st, u, delta, dt);
+            if (live) live = march_advance<false>(p.m, ry, st, u, delta, dt);
             if (!__any_sync(0xffffffffu, live)) break;
             if (slot == kSlots) {
                 uint32_t c = 0;
@@ -150,7 +151,7 @@ __global__ void __launch_bounds__(128, kDist ? 6 : 4) record_kernel(const __grid
                 const float t = df_float(st.t);
                 const float sigma = expf(f[0]);
                 const float trans = expf(-sigma * delta);
-                const float w = T * (1.0f - trans);
+                const float w = fmul(T, fsub(1.0f, trans));
                 const float T_next = T * trans;
                 float gs;
                 if constexpr (kDist) {
@@ -174,7 +175,7 @@ __global__ void __launch_bounds__(128, kDist ? 6 : 4) record_kernel(const __grid
                 p.chunk_n[(size_t)chunk * 32 + lane] = slot + 1;
                 T = T_next;
                 if (T < p.m.opts.t_term) live = false;
-                else march_after_sample(p.m, st, dt);
+                else march_after_sample<false>(p.m, st, dt);
             }
             ++slot;
         }

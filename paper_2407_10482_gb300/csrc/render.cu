@@ -205,10 +205,13 @@ __global__ void grid_indices_kernel(const __grid_constant__ IndexParams p) {
 int32_t make_grid(const ngprt_scene* s, Grid& g, const char* fn);
 int32_t make_occ(const ngprt_occ* o, OccView& v, const char* fn);
 
-template <int L>
-void launch_march(int dt, const MarchParams& p, dim3 grid, cudaStream_t st) {
-    launch_march_kernel<L, NGPRT_AGG_SEPARATE_V>(dt, p, grid, st);
-}
+// render_l<L>.cu
+void launch_march_l1(int dt, const MarchParams& p, dim3 grid, cudaStream_t st);
+void launch_march_l2(int dt, const MarchParams& p, dim3 grid, cudaStream_t st);
+void launch_march_l3(int dt, const MarchParams& p, dim3 grid, cudaStream_t st);
+void launch_march_l4(int dt, const MarchParams& p, dim3 grid, cudaStream_t st);
+void launch_march_l8(int dt, const MarchParams& p, dim3 grid, cudaStream_t st);
+void launch_march_l16(int dt, const MarchParams& p, dim3 grid, cudaStream_t st);
 
 template <int L>
 void launch_targets(int dt, const MarchParams& p, dim3 grid, cudaStream_t st, float* targets) {
@@ -230,12 +233,12 @@ bool march_supports(int L) { return march_supports(L, NGPRT_AGG_SEPARATE_V); }
 int32_t launch_march_any(int L, int dt, int agg, const MarchParams& p, dim3 grid, cudaStream_t st) {
     if (agg != NGPRT_AGG_SEPARATE_V) return launch_march_agg(L, dt, agg, p, grid, st);
     switch (L) {
-        case 1: launch_march<1>(dt, p, grid, st); break;
-        case 2: launch_march<2>(dt, p, grid, st); break;
-        case 3: launch_march<3>(dt, p, grid, st); break;
-        case 4: launch_march<4>(dt, p, grid, st); break;
-        case 8: launch_march<8>(dt, p, grid, st); break;
-        case 16: launch_march<16>(dt, p, grid, st); break;
+        case 1: launch_march_l1(dt, p, grid, st); break;
+        case 2: launch_march_l2(dt, p, grid, st); break;
+        case 3: launch_march_l3(dt, p, grid, st); break;
+        case 4: launch_march_l4(dt, p, grid, st); break;
+        case 8: launch_march_l8(dt, p, grid, st); break;
+        case 16: launch_march_l16(dt, p, grid, st); break;
         default: set_error("march kernel not built for L=%d", L); return NGPRT_ERR_UNSUPPORTED;
     }
     return NGPRT_OK;

@@ -157,3 +157,25 @@ def test_lane_groups_render_the_one_lane_rays(n, dtype):
         assert torch.equal(part["stats"], full["stats"][:n])
         torch.testing.assert_close(part["state"], full["state"][:n], rtol=2e-6, atol=2e-6)
         torch.testing.assert_close(part["rgb"], full["rgb"][:n], rtol=0, atol=2e-6)
+
+
+@pytest.mark.parametrize("lattice_snap", [False, True])
+@pytest.mark.parametrize("n", [33, 40000, 75001, 140001])
+@pytest.mark.parametrize("dtype", ["F32", "F16", "BF16"])
+def test_medium_batches_render_the_rays_of_a_full_one(n, dtype, lattice_snap):
+    """Batches below a full GPU (march kernel with more registers, or lane groups, and
+    neither where the samples stay on a lattice at few rays) against the same rays in a
+    batch that fills it, with the bounds of the lane groups above."""
+    from paper_2407_10482_gb300 import ngprt as ng
+    cfg = S.small_config(blob_std=(0.05, 0.15))
+    sc = S.make_scene(cfg)
+    ds = ng.DeviceScene(cfg, sc.tables, sc.coarse, sc.mlp_w, table_dtype=getattr(ng, dtype))
+    rend = ng.Renderer(ds, ng.DeviceOcc(sc.occ, cfg.R_O, cfg.n_occ_levels))
+    o, d = S.random_rays(300000, 4, cfg.bounded)
+    o, d = torch.as_tensor(o).cuda(), torch.as_tensor(d).cuda()
+    opts = S.default_options(cfg, lattice_snap=lattice_snap)
+    full = rend.render(opts, rays_o=o, rays_d=d, stats=True, state=True)
+    part = rend.render(opts, rays_o=o[:n].contiguous(), rays_d=d[:n].contiguous(), stats=True, state=True)
+    assert torch.equal(part["stats"], full["stats"][:n])
+    torch.testing.assert_close(part["state"], full["state"][:n], rtol=2e-6, atol=2e-6)
+    torch.testing.assert_close(part["rgb"], full["rgb"][:n], rtol=0, atol=2e-6)
