@@ -35,8 +35,17 @@
 // with 8 steps a chunk and each lane adding its rows by itself, 6.4 with 16 steps, 4.8 with
 // the lanes in pairs; levels and logits in kernels of their own, each with the blocks its
 // registers allow, gave the rest.  The march is bound by the same 180 G sectors a second
-// that its gathers take from L2.  The regulariser at the same rays: 1.9 + 2.8 ms in place
-// of 29.3.
+// that its gathers take from L2.
+//
+// The regulariser takes records up to kDistRecordRays rays: 2^16 camera pixels of the hd
+// scene, forward and reverse pass, 3.0 ms in place of 10.4; 8 levels 1.66 in place of 3.30.
+// Beyond, its reverse pass stays in one kernel.  The gradients of a row are many small
+// terms of both signs there, and what a float accumulator keeps of them depends on how
+// they are grouped: at 2^18 rays the one-kernel form is 4e-5 of the coarse gradient away
+// from sums in 64 bits and the run sums 3e-6, so that the two forms differ by up to 4e-5,
+// more than FP32 results of one call are to move here; at 2^16 by 8e-6.  (2^18 rays took
+// 6.5 ms by run sums in place of 36; 10.6 with the dense levels added sample by sample in
+// the given ray order, which left 2.2e-5 on 8 levels.)
 #pragma once
 #include <string.h>
 
@@ -49,6 +58,7 @@ constexpr int kRunChunks = 8;   // chunks provided per run of 32 rays, at most
 constexpr size_t kRecordBytes = (size_t)3 << 30;  // and of all runs, at most
 constexpr int64_t kRecordRays = 1 << 18;   // rays per pass (records of more are processed in turn)
 constexpr int64_t kRecordMinRays = 4096;   // fewer rays take the one-kernel form
+constexpr int64_t kDistRecordRays = 1 << 16;  // more rays of the regulariser take the one-kernel form
 constexpr int kMaxBins = 1 << 16;
 
 template <int L, bool kDist>
@@ -554,7 +564,7 @@ inline bool plane_serves(const ngprt_scene* s) {
 
 // Bytes that the records of a reverse pass take (0: the pass keeps none).
 inline size_t record_scratch_bytes(int L, bool dist, int64_t n_rays) {
-    if (n_rays < kRecordMinRays || n_rays > 0x7FFFFFFF) return 0;
+    if (n_rays < kRecordMinRays || n_rays > (dist ? kDistRecordRays : 0x7FFFFFFF)) return 0;
     return record_layout(L, dist, n_rays).bytes;
 }
 
