@@ -467,7 +467,8 @@ size_t ngprt_distortion_backward_workspace_bytes(const ngprt_scene* scene, const
                                                  int64_t n_rays);
 /* Bytes with which ngprt_distortion_backward is fastest, as
  * ngprt_render_backward_scratch_bytes (any smaller workspace the call accepts without
- * them is still accepted). */
+ * them is still accepted, and so is a g_coarse off 16-byte alignment, which takes the form
+ * that adds every sample by itself). */
 size_t ngprt_distortion_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
                                                int64_t n_rays);
 int32_t ngprt_distortion_loss(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,

@@ -244,7 +244,11 @@ static int32_t run_distortion(bool backward, const ngprt_scene* scene, const ngp
     }
     void* records = nullptr;
     float* g_plane = nullptr;
-    if (workspace && plane_serves(scene) && !lattice(p.m)) {
+    // the scatter of the records adds 16 bytes of a coarse row at a time; a gradient that
+    // starts anywhere else (a view into a flat buffer) takes the one-kernel form's single
+    // floats
+    const bool wide = !backward || ((uintptr_t)g_coarse & 15) == 0;
+    if (workspace && plane_serves(scene) && !lattice(p.m) && wide) {
         const int64_t entries = ngprt_table_entries(scene);
         const size_t plane = plane_layout(entries, backward ? 0 : n_rays, backward).bytes;
         const size_t rec = backward ? record_scratch_bytes(L, true, n_rays) : 0;

@@ -1,0 +1,41 @@
+"""Calls that take the general route because of their alignment, size or scene, against
+the form that serves every call."""
+import ctypes as C
+
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from test_gpu_records import _close, _setup
+
+pytestmark = pytest.mark.gpu
+
+
+def _ptr(t):
+    return None if t is None else C.c_void_p(t.data_ptr())
+
+
+def _distortion_gradients(L, n, pixels, offset=0, **kw):
+    """(gradients of the binding's call, of the C entry without scratch); g_coarse of the
+    first starts `offset` floats into a flat buffer."""
+    ng, ds, occ, opts, rays, src = _setup(L, n, pixels, **kw)
+    ro = ng.render_opts(opts)
+    state = torch.empty(n, 4, device="cuda")
+    ng.ngprt_distortion_loss(ds.struct, occ.struct, *src, n, ro, 1.0, state)
+    flat = torch.zeros(ds.coarse.numel() + offset, device="cuda")
+    got = [torch.zeros_like(ds.tables), flat[offset:].view_as(ds.coarse)]
+    ref = [torch.zeros_like(t) for t in (ds.tables, ds.coarse)]
+    ng.ngprt_distortion_backward(ds.struct, occ.struct, *src, n, ro, state, 1.0 / n, *got)
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert ng.lib().ngprt_distortion_backward(
+        C.byref(ds.struct), C.byref(occ.struct), src[0], src[1], _ptr(src[2]), _ptr(src[3]), _ptr(src[4]), n, C.byref(ro),
+        _ptr(state), C.c_float(1.0 / n), _ptr(ref[0]), _ptr(ref[1]), None, None, None, 0, st) == 0
+    return got, ref
+
+
+@pytest.mark.parametrize("offset", [0, 1, 2, 4])
+@pytest.mark.parametrize("L", [2, 8, 16])
+def test_distortion_gradient_in_a_flat_buffer(L, offset):
+    """Bounds of the records' tests: the same FP32 terms in another order."""
+    for a, b in zip(*_distortion_gradients(L, 4096 + 33, True, offset)):
+        _close(a, b)
