@@ -538,6 +538,7 @@ class Renderer:
         self.scene, self.occ, self.device = scene, occ, device
         self._ws = None
         self._bws = None  # the reverse pass's workspace
+        self._no_scratch = float("inf")  # scratch of so many bytes could not be had
 
     def workspace(self, n_rays: int):
         need = ngprt_render_workspace_bytes(self.scene.struct, n_rays)
@@ -611,15 +612,22 @@ def _renderer_backward(self, opts, state, d_rgb, d_depth, d_opacity, g_tables, g
         cam_arr, n_cams = None, 0
         n = rays_o.shape[0]
     ro = render_opts(opts)
+    need = ngprt_render_backward_workspace_bytes(self.scene.struct, ro, n)
     best = ngprt_render_backward_scratch_bytes(self.scene.struct, ro, n)
-    if self._bws is None or self._bws.numel() < best:
-        self._bws = None  # given back before a larger one is asked for
-        self._bws = _scratch(best, self.scene.tables)
-    if self._bws is None:
-        need = ngprt_render_backward_workspace_bytes(self.scene.struct, ro, n)
-        self._bws = torch.empty(need, dtype=torch.uint8, device=self.device)
+    # the records' scratch (up to 3 GB) is the call's own: the caching allocator hands it to
+    # other tensors between calls, and two streams never share it.  A size that could not be
+    # had is not asked for again (each failure empties the allocator's cache).
+    ws = None
+    if need < best < self._no_scratch:
+        ws = _scratch(best, self.scene.tables)
+        if ws is None and not torch.cuda.is_current_stream_capturing():
+            self._no_scratch = best
+    if ws is None:
+        if self._bws is None or self._bws.numel() < need:
+            self._bws = torch.empty(need, dtype=torch.uint8, device=self.device)
+        ws = self._bws
     ngprt_render_backward(self.scene.struct, self.occ.struct, cam_arr, n_cams, pixel_ids, rays_o, rays_d, n,
-                          ro, state, d_rgb, d_depth, d_opacity, g_tables, g_coarse, g_mlp, self._bws,
+                          ro, state, d_rgb, d_depth, d_opacity, g_tables, g_coarse, g_mlp, ws,
                           g_attn_inv=g_attn_inv, g_agg_mlp=g_agg_mlp)
 
 
