@@ -165,10 +165,12 @@ def _stream(stream=None) -> int | None:
     return stream.cuda_stream
 
 
-def _scratch(nbytes: int, like: torch.Tensor, stream=None):
+def _scratch(nbytes: int, like, stream=None):
     """Scratch of a call that also runs without any: a block of torch's caching allocator
-    on the call's stream, or None (nothing to gain, no memory left, a capture running)."""
-    if not nbytes:
+    on the call's stream and on the device of its output `like` (a tensor, or an address on
+    the current device), or None: nothing to gain, no output (which the call reports), a
+    stream that torch cannot allocate on, no memory left, a capture running."""
+    if not nbytes or like is None or not (stream is None or isinstance(stream, torch.cuda.Stream)):
         return None
     if stream is not None:
         with torch.cuda.stream(stream):
@@ -176,7 +178,8 @@ def _scratch(nbytes: int, like: torch.Tensor, stream=None):
     if torch.cuda.is_current_stream_capturing():
         return None
     try:
-        return torch.empty(nbytes, dtype=torch.uint8, device=like.device)
+        return torch.empty(nbytes, dtype=torch.uint8,
+                           device=like.device if isinstance(like, torch.Tensor) else "cuda")
     except torch.OutOfMemoryError:
         return None
 

@@ -68,3 +68,62 @@ def test_a_capture_keeps_the_workspace(renderer, monkeypatch):
     renderer.room = True
     _backward(renderer)
     assert renderer.given[-1] == BEST
+
+
+class _Stream:
+    """A stream of another library: a handle and nothing else."""
+    cuda_stream = 7
+
+
+@pytest.fixture
+def entry(monkeypatch):
+    """ngprt_occupancy_from_density on a stand-in library that wants scratch; returns the
+    arguments of the native calls, and the devices of the allocations."""
+    calls, devices = [], []
+
+    class Lib:
+        def ngprt_last_error(self):
+            return b"occ_out is NULL"
+
+        def __getattr__(self, name):
+            def call(*a):
+                calls.append(a)
+                return 0 if a[4] else -1
+            return call
+
+    empty = torch.empty
+
+    def alloc(n, dtype=None, device=None):
+        devices.append(str(device))
+        return empty(n, dtype=dtype)
+
+    monkeypatch.setattr(ng, "lib", lambda: Lib())
+    for name in ("ngprt_density_scratch_bytes", "ngprt_occupancy_from_density_scratch_bytes"):
+        monkeypatch.setattr(ng, name, lambda *a: 64, raising=False)
+    ptr = ng._ptr
+    monkeypatch.setattr(ng, "_ptr", lambda t: t.data_ptr() if isinstance(t, torch.Tensor) else ptr(t))
+    monkeypatch.setattr(torch, "empty", alloc)
+    monkeypatch.setattr(torch.cuda, "is_current_stream_capturing", lambda: False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: _Stream)
+    return calls, devices
+
+
+def _density(out, **kw):
+    ng.ngprt_occupancy_from_density(ng.ngprt_scene(), ng.ngprt_render_opts(), 64, 1.0, out, **kw)
+
+
+def test_outputs_given_as_addresses(entry):
+    calls, devices = entry
+    _density(4096)
+    assert devices == ["cuda"] and calls[0][4] == 4096
+
+
+def test_a_missing_output_is_the_library_s_error(entry):
+    with pytest.raises(ng.NgprtError, match="occ_out is NULL"):
+        _density(None)
+
+
+def test_streams_that_torch_cannot_allocate_on(entry):
+    calls, devices = entry
+    _density(4096, stream=_Stream)
+    assert devices == [] and calls[0][-1] == 7
