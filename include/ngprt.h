@@ -268,13 +268,15 @@ int32_t ngprt_occupancy_visibility(const ngprt_scene* scene, const ngprt_occ* oc
 /*
  * The passes that read the density path alone (ngprt_occupancy_from_density,
  * ngprt_occupancy_visibility, ngprt_distortion_loss) in forms with a workspace: with
- * ngprt_density_scratch_bytes(scene, n_rays) bytes (n_rays = 0 for
- * ngprt_occupancy_from_density_ws; 0 bytes where the scene has no faster form) they copy
- * the tables' density channel there first and, for camera pixel lists, take the rays in
- * pixel-tile order.  The results are those of the forms without; a NULL or smaller
- * workspace gives exactly those forms.
+ * ngprt_density_scratch_bytes(scene, n_rays) bytes, or
+ * ngprt_occupancy_from_density_scratch_bytes(scene, R), they copy the tables' density
+ * channel there first and, for camera pixel lists, take the rays in pixel-tile order.  The
+ * results are those of the forms without; a NULL or smaller workspace gives exactly those
+ * forms, and so does any where the query returns 0 (the scene has no faster form, or the
+ * call is too small for the copy to pay).
  */
 size_t ngprt_density_scratch_bytes(const ngprt_scene* scene, int64_t n_rays);
+size_t ngprt_occupancy_from_density_scratch_bytes(const ngprt_scene* scene, int32_t R);
 int32_t ngprt_occupancy_from_density_ws(const ngprt_scene* scene, const ngprt_render_opts* opts, int32_t R,
                                         float sigma_thr, uint8_t* occ_out, float* sigma_out, void* workspace,
                                         size_t ws_bytes, void* stream);

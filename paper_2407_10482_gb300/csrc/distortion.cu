@@ -248,7 +248,7 @@ static int32_t run_distortion(bool backward, const ngprt_scene* scene, const ngp
     // starts anywhere else (a view into a flat buffer) takes the one-kernel form's single
     // floats
     const bool wide = !backward || ((uintptr_t)g_coarse & 15) == 0;
-    if (workspace && plane_serves(scene) && !lattice(p.m) && wide) {
+    if (workspace && (backward ? plane_serves(scene) : plane_pays(scene, n_rays)) && !lattice(p.m) && wide) {
         const int64_t entries = ngprt_table_entries(scene);
         const size_t plane = plane_layout(entries, backward ? 0 : n_rays, backward).bytes;
         const size_t rec = backward ? record_scratch_bytes(L, true, n_rays) : 0;

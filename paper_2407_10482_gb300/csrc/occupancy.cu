@@ -39,8 +39,13 @@ static bool pow2_in(int32_t R) { return R >= 2 && R <= 1024 && (R & (R - 1)) == 
 using namespace ngprt;
 
 extern "C" size_t ngprt_density_scratch_bytes(const ngprt_scene* scene, int64_t n_rays) {
-    if (n_rays < 0 || !plane_serves(scene)) return 0;
+    if (!plane_pays(scene, n_rays)) return 0;
     return plane_layout(ngprt_table_entries(scene), n_rays).bytes;
+}
+
+extern "C" size_t ngprt_occupancy_from_density_scratch_bytes(const ngprt_scene* scene, int32_t R) {
+    if (!pow2_in(R) || !plane_pays_voxels(scene, R)) return 0;
+    return plane_layout(ngprt_table_entries(scene), 0).bytes;
 }
 
 extern "C" int32_t ngprt_occupancy_from_density(const ngprt_scene* scene, const ngprt_render_opts* opts, int32_t R,
@@ -72,7 +77,8 @@ extern "C" int32_t ngprt_occupancy_from_density_ws(const ngprt_scene* scene, con
         return cuda_status(fn);
     }
     const bool built = scene->L <= 4 || scene->L == 8 || scene->L == 16;
-    if (built && workspace && plane_serves(scene) && ws_bytes >= ngprt_density_scratch_bytes(scene, 0)) {
+    const size_t best = ngprt_occupancy_from_density_scratch_bytes(scene, R);
+    if (built && workspace && best && ws_bytes >= best) {
         MarchParams m;
         memset(&m, 0, sizeof m);
         m.g = p.g;
@@ -127,8 +133,8 @@ extern "C" int32_t ngprt_occupancy_visibility_ws(const ngprt_scene* scene, const
         return cuda_status(fn);
     }
     const bool built = scene->L <= 4 || scene->L == 8 || scene->L == 16;
-    if (built && workspace && plane_serves(scene) && !lattice(p) &&
-        ws_bytes >= ngprt_density_scratch_bytes(scene, n_rays))
+    const size_t best = ngprt_density_scratch_bytes(scene, n_rays);
+    if (built && workspace && best && ws_bytes >= best && !lattice(p))
         density_scratch(p, ngprt_table_entries(scene), true, workspace, st);
     switch (scene->L) {
         case 1: launch_visibility<1, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, grid, w_thr, R, vis, st); break;

@@ -562,6 +562,26 @@ inline bool plane_serves(const ngprt_scene* s) {
            ngprt_table_entries(s) >= kPlaneMinEntries;
 }
 
+// Whether the plane's copy (hd, 6.1 M rows: 45 us; 42 M rows: 250 us) pays for a forward
+// pass over rays: from 4096 rays on, and a ray for every 2000 rows, for stacks of up to 4
+// levels, whose samples gain less, for every 140.  us without and with the plane,
+// visibility pass: hd, 1 ray 97 and 152, 1000 random pixels 1072 and 1038, 4096 1323 and
+// 889; 42 M rows, 1 ray 97 and 352, 6912 pixels of an image 1183 and 1332, 65536 1668 and
+// 1399; 2 levels, 1 M rows, 4096 free rays 239 and 250, 65536 344 and 327.  (Where every ray
+// ends after some 14 samples the copy does not pay back at 4096 rays: 174 and 219.)
+inline bool plane_pays(const ngprt_scene* s, int64_t n_rays) {
+    return plane_serves(s) && n_rays >= kRecordMinRays &&
+           n_rays >= ngprt_table_entries(s) / (s->L <= 4 ? 140 : 2000);
+}
+
+// The same for a density at R^3 voxels: a voxel for every 32 rows, and enough work for
+// another launch.  hd: 32^3 32 and 56 us, 64^3 122 and 81, 128^3 698 and 263; 42 M rows:
+// 64^3 234 and 290, 128^3 1487 and 493; 2 levels: 64^3 17 and 19, 128^3 82 and 54.
+inline bool plane_pays_voxels(const ngprt_scene* s, int32_t R) {
+    const int64_t n = (int64_t)R * R * R;
+    return plane_serves(s) && n >= ngprt_table_entries(s) / 32 && n * s->L > 1 << 20;
+}
+
 // Bytes that the records of a reverse pass take (0: the pass keeps none).
 inline size_t record_scratch_bytes(int L, bool dist, int64_t n_rays) {
     if (n_rays < kRecordMinRays || n_rays > (dist ? kDistRecordRays : 0x7FFFFFFF)) return 0;

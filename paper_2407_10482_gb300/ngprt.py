@@ -71,6 +71,7 @@ _SIGS = {
     "ngprt_occupancy_visibility": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, C.c_float,
                                                C.c_int32, _P, _P]),
     "ngprt_density_scratch_bytes": (C.c_size_t, [_P, C.c_int64]),
+    "ngprt_occupancy_from_density_scratch_bytes": (C.c_size_t, [_P, C.c_int32]),
     "ngprt_occupancy_from_density_ws": (C.c_int32, [_P, _P, C.c_int32, C.c_float, _P, _P, _P, C.c_size_t, _P]),
     "ngprt_occupancy_visibility_ws": (C.c_int32, [_P, _P, _P, C.c_int32, _P, _P, _P, C.c_int64, _P, C.c_float,
                                                   C.c_int32, _P, _P, C.c_size_t, _P]),
@@ -215,7 +216,7 @@ def ngprt_coarse_channels(L: int, aggregation: int) -> int:
 
 
 def ngprt_occupancy_from_density(scene, opts, R, sigma_thr, occ_out, sigma_out=None, stream=None) -> None:
-    ws = _scratch(ngprt_density_scratch_bytes(scene, 0), occ_out, stream)
+    ws = _scratch(ngprt_occupancy_from_density_scratch_bytes(scene, R), occ_out, stream)
     _check("ngprt_occupancy_from_density", lib().ngprt_occupancy_from_density_ws(
         C.byref(scene), C.byref(opts), R, sigma_thr, _ptr(occ_out), _ptr(sigma_out), _ptr(ws),
         ws.numel() if ws is not None else 0, _stream(stream)))
@@ -265,6 +266,10 @@ def ngprt_distortion_backward_scratch_bytes(scene, opts, n_rays) -> int:
 
 def ngprt_density_scratch_bytes(scene, n_rays) -> int:
     return int(lib().ngprt_density_scratch_bytes(C.byref(scene), n_rays))
+
+
+def ngprt_occupancy_from_density_scratch_bytes(scene, R) -> int:
+    return int(lib().ngprt_occupancy_from_density_scratch_bytes(C.byref(scene), R))
 
 
 def ngprt_mean_samples(ray_stats, n_rays, out, stream=None) -> None:

@@ -39,3 +39,30 @@ def test_distortion_gradient_in_a_flat_buffer(L, offset):
     """Bounds of the records' tests: the same FP32 terms in another order."""
     for a, b in zip(*_distortion_gradients(L, 4096 + 33, True, offset)):
         _close(a, b)
+
+
+@pytest.mark.parametrize("sparse", [False, True])
+@pytest.mark.parametrize("attn_mode", [0, 2])
+@pytest.mark.parametrize("L,R", [(2, 128), (4, 128), (8, 64), (16, 64)])
+def test_occupancy_on_the_density_plane_of_large_calls(L, R, attn_mode, sparse):
+    """The density channel's sums keep their order: equal bit for bit, on the dense coarse
+    grid and on its block-sparse form."""
+    n = 40000
+    ng, ds, occ, opts, rays, src = _setup(L, n, True, attn_mode=attn_mode)
+    if sparse:
+        ds.sparsify_coarse(occ)
+    ro, lib = ng.render_opts(opts), ng.lib()
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert ng.ngprt_occupancy_from_density_scratch_bytes(ds.struct, R) > 0
+    assert ng.ngprt_density_scratch_bytes(ds.struct, n) > 0
+    o = [torch.empty(R ** 3, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    sg = [torch.empty(R ** 3, device="cuda") for _ in range(2)]
+    ng.ngprt_occupancy_from_density(ds.struct, ro, R, 1.0, o[0], sg[0])
+    assert lib.ngprt_occupancy_from_density(C.byref(ds.struct), C.byref(ro), R, C.c_float(1.0), _ptr(o[1]), _ptr(sg[1]),
+                                            st) == 0
+    assert torch.equal(o[0], o[1]) and torch.equal(sg[0], sg[1])
+    v = [torch.zeros(R ** 3, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    ng.ngprt_occupancy_visibility(ds.struct, occ.struct, *src, n, ro, 1e-3, R, v[0])
+    assert lib.ngprt_occupancy_visibility(C.byref(ds.struct), C.byref(occ.struct), src[0], src[1], _ptr(src[2]), None,
+                                          None, n, C.byref(ro), C.c_float(1e-3), R, _ptr(v[1]), st) == 0
+    assert torch.equal(v[0], v[1]) and int(v[0].sum()) > 0
