@@ -31,6 +31,15 @@ struct MarchBwdParams {
     const int32_t* n_list;    // their count (device)
 };
 
+// Entry `at` of a list of n rays, taken in scattered order (at times a prime above every n,
+// modulo n).  The list fills in the order in which the rays ran out of records; neighbours
+// in it are neighbours in the image, and their additions to the same few rows wait for one
+// another (hd model on a full grid, 474 samples a ray, 2^18 rays: 684 ms in the list's
+// order, 515 scattered, 522 with no records; 2 levels: 90, 66 and 68 ms).
+__device__ __forceinline__ int2 listed_ray(const int2* list, int n, int at) {
+    return list[(uint64_t)at * 2654435761ull % (uint64_t)n];
+}
+
 // The ray `ray` of the batch set up for its march; false when its interval is empty.
 __device__ __forceinline__ bool ray_setup_at(const MarchParams& p, int64_t ray, Ray& ry) {
     float o[3];
@@ -344,8 +353,9 @@ __global__ void __launch_bounds__(128, NGPRT_BWD_MIN_BLOCKS) march_backward_kern
         const int at = blockIdx.x * blockDim.x + threadIdx.x;
         live = at < *p.n_list;
         if (live) {
-            ray = p.list[at].x;
-            skip = p.list[at].y;
+            const int2 e = listed_ray(p.list, *p.n_list, at);
+            ray = e.x;
+            skip = e.y;
             live = ray_setup_at(p.m, ray, ry);
         }
     } else {

@@ -114,8 +114,9 @@ __global__ void __launch_bounds__(128) distortion_backward_kernel(const __grid_c
     if (p.list) {
         const int at = blockIdx.x * blockDim.x + threadIdx.x;
         if (at >= *p.n_list) return;
-        ray = p.list[at].x;
-        skip = p.list[at].y;
+        const int2 e = listed_ray(p.list, *p.n_list, at);
+        ray = e.x;
+        skip = e.y;
         hit = ray_setup_at(p.m, ray, ry);
     } else if (!ray_setup(p.m, ray, ry, hit)) {
         return;

@@ -6,7 +6,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
-from test_gpu_records import _close, _setup
+from test_gpu_records import _close, _render_gradients, _setup
 
 pytestmark = pytest.mark.gpu
 
@@ -66,3 +66,21 @@ def test_occupancy_on_the_density_plane_of_large_calls(L, R, attn_mode, sparse):
     assert lib.ngprt_occupancy_visibility(C.byref(ds.struct), C.byref(occ.struct), src[0], src[1], _ptr(src[2]), None,
                                           None, n, C.byref(ro), C.c_float(1e-3), R, _ptr(v[1]), st) == 0
     assert torch.equal(v[0], v[1]) and int(v[0].sum()) > 0
+
+
+def _overflow(L, n, pixels):
+    """More samples a ray than the records hold (128, or 44 for 2^18 rays of 16 levels):
+    the rest comes from the one-kernel form, whose list is taken in scattered order."""
+    step = 2.0 * 3 ** 0.5 / 128.0 / 8.0
+    _render_gradients(L, n, pixels, step_base=step, max_samples=512, max_march=4096, t_term=0.0)
+
+
+@pytest.mark.parametrize("L,n,pixels", [(1, 4097, True), (4, 4096, False), (8, 5001, True), (16, 1 << 18, True)])
+def test_rays_beyond_the_records_room(L, n, pixels):
+    _overflow(L, n, pixels)
+
+
+def test_distortion_beyond_the_records_room():
+    step = 2.0 * 3 ** 0.5 / 128.0 / 8.0
+    for a, b in zip(*_distortion_gradients(8, 5001, True, step_base=step, max_samples=512, max_march=4096, t_term=0.0)):
+        _close(a, b)
