@@ -380,7 +380,7 @@ const int32_t* bin_rays(const MarchParams& m, uint32_t* bins, int32_t* perm, cud
 // Eq. 8's reverse march: by records where the scratch is there, else in one kernel.
 template <int L>
 static void launch_bwd_l(const MarchBwdParams& p, dim3 grid, void* scratch, cudaStream_t st) {
-    if (!scratch || lattice(p.m)) {
+    if (!scratch || lattice(p.m) || !records_pay(L, p.m)) {
         launch_bwd<L, NGPRT_AGG_SEPARATE_V>(p, grid, st);
         return;
     }

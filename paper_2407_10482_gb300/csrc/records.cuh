@@ -17,8 +17,8 @@
 // so a thread that walks a ray's records at one level needs 16 sums, and adds them to the
 // 8 rows when the cell changes or the records end.
 //
-// Kernel 1 (record_kernel): warps take runs of 32 rays (in pixel-tile order for camera
-// pixels: the rays are binned by 32 x 32 pixel tile first) and march them together; each
+// Kernel 1 (record_kernel): warps take runs of 32 rays (large lists of camera pixels in
+// pixel-tile order: the rays are binned by 32 x 32 pixel tile first) and march them together; each
 // step of the warp is one slot of a chunk of kSlots steps x 32 lanes, taken from a
 // counter when the previous chunk is full.  Record fields are lane-contiguous:
 //     u (3), gs, w, then omega, beta, sigma^l, q^l per level   (kDist: u, gs, omega, sigma^l)
@@ -58,6 +58,21 @@ constexpr int kRunChunks = 8;   // chunks provided per run of 32 rays, at most
 constexpr size_t kRecordBytes = (size_t)3 << 30;  // and of all runs, at most
 constexpr int64_t kRecordRays = 1 << 18;   // rays per pass (records of more are processed in turn)
 constexpr int64_t kRecordMinRays = 4096;   // fewer rays take the one-kernel form
+// Render's records are taken in pixel-tile order from so many rays on.  Below, neighbours
+// add to the same rows at the same time and wait for one another (us without records, in
+// tile order and in the given order: 2 levels, 16384 random pixels 503, 806 and 555; 16
+// levels, 32768 2890, 2122 and 1963); above, their gathers meet in L1 (16 levels, 2^17
+// 10622, 4559 and 5301).  The regulariser's records never are: 16 levels, 2^16 1892 and
+// 1681; 2 levels, 16384 747 and 473, without records 516.
+constexpr int64_t kBinRays = 1 << 16;
+// Pixel lists of 2 and 4 levels take the one-kernel form up to so many rays: it adds whole
+// rows of their coarse grid at a time, and its latency hides what records save (16384
+// pixels: 2 levels 503 us against 555, 4 levels 603 against 669, bounded 488 against 523;
+// 65536: 1266 against 863).
+constexpr int64_t kFewLevelRays = 1 << 15;
+inline bool records_pay(int L, const MarchParams& m) {
+    return m.mode != 1 || (L != 2 && L != 4) || m.n_rays > kFewLevelRays;
+}
 constexpr int64_t kDistRecordRays = 1 << 16;  // more rays of the regulariser take the one-kernel form
 constexpr int kMaxBins = 1 << 16;
 
@@ -503,6 +518,7 @@ __device__ __forceinline__ uint32_t bin_of(const BinParams& p, int64_t i) {
 struct RecLayout {
     size_t counters, perm, bins, list, chunk_ray, chunk_n, rec, bytes;
     uint32_t max_chunks;
+    bool order;  // room for the pixel-tile order
 };
 
 inline RecLayout record_layout(int L, bool dist, int64_t n_rays) {
@@ -514,8 +530,9 @@ inline RecLayout record_layout(int L, bool dist, int64_t n_rays) {
     a.max_chunks = (uint32_t)(want < room ? want : room);
     size_t at = 0;
     a.counters = at; at += 256;
-    a.perm = at; at += up((size_t)n_rays * sizeof(int32_t));
-    a.bins = at; at += up((size_t)kMaxBins * sizeof(uint32_t));
+    a.order = !dist && n_rays >= kBinRays;
+    a.perm = at; at += a.order ? up((size_t)n_rays * sizeof(int32_t)) : 0;
+    a.bins = at; at += a.order ? up((size_t)kMaxBins * sizeof(uint32_t)) : 0;
     a.list = at; at += up((size_t)pass * sizeof(int2));
     a.chunk_ray = at; at += up((size_t)a.max_chunks * 32 * sizeof(int32_t));
     a.chunk_n = at; at += up((size_t)a.max_chunks * 32 * sizeof(int32_t));
@@ -606,7 +623,9 @@ void launch_records(RecParams p, void* scratch, cudaStream_t st, Rest rest) {
     p.chunk_n = reinterpret_cast<int32_t*>(base + a.chunk_n);
     p.rec = reinterpret_cast<float*>(base + a.rec);
     p.max_chunks = a.max_chunks;
-    p.perm = bin_rays(p.m, reinterpret_cast<uint32_t*>(base + a.bins), reinterpret_cast<int32_t*>(base + a.perm), st);
+    p.perm = nullptr;
+    if (a.order)
+        p.perm = bin_rays(p.m, reinterpret_cast<uint32_t*>(base + a.bins), reinterpret_cast<int32_t*>(base + a.perm), st);
     static int cache1[16] = {0}, cache2[16] = {0}, cache3[16] = {0};
     const unsigned g1 = resident_grid(record_kernel<L, kDist>, cache1),
                    g2 = resident_grid(scatter_levels_kernel<L, kDist>, cache2),

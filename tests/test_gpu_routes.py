@@ -84,3 +84,20 @@ def test_distortion_beyond_the_records_room():
     step = 2.0 * 3 ** 0.5 / 128.0 / 8.0
     for a, b in zip(*_distortion_gradients(8, 5001, True, step_base=step, max_samples=512, max_march=4096, t_term=0.0)):
         _close(a, b)
+
+
+@pytest.mark.parametrize("L", [2, 4])
+def test_pixel_lists_of_few_levels_by_records(L):
+    """2 and 4 levels take pixel lists by records above 2^15 rays."""
+    _render_gradients(L, (1 << 15) + 33, True)
+
+
+@pytest.mark.parametrize("L", [1, 4, 8, 16])
+def test_pixel_lists_in_tile_order(L):
+    """Lists of at least 2^16 pixels are recorded in pixel-tile order."""
+    _render_gradients(L, (1 << 16) + 33, True)
+
+
+@pytest.mark.parametrize("pixels", [True, False])
+def test_more_rays_than_one_pass_of_records(pixels):
+    _render_gradients(1, (1 << 18) + 4129, pixels)
