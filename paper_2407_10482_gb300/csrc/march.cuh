@@ -1131,10 +1131,10 @@ __global__ void __launch_bounds__(128, kBlocks) march_kernel(const __grid_consta
 // gathered at the same time; the transmittances then pass along the group in sample
 // order, so every sum and decision is that of the one-lane march.  A ray that terminates
 // inside a group of samples drops the later ones (their points are not counted).
-// Bound by that chain's latency: a 64 x 64 call of the small scene 323 -> 79 us, 50001
-// free rays of an 8-level scene (G = 2) 832 -> 695 us for the march.
-// Three blocks per SM: 168 registers, no spills (79 us; at 4 and 5 blocks 76-82 and 83,
-// but 50001 rays 3% and 4% slower).
+// Bound by that chain's latency: a 64 x 64 call of the small scene 341 -> 75 us, 4096
+// random pixels of the hd scene 1957 -> 325 us.
+// Three blocks per SM: 168 registers, no spills (small scene 79 us; at 4 and 5 blocks 76-82
+// and 83).
 template <int L, int DT, int AGG>
 __global__ void __launch_bounds__(128, 3)
     march_group_kernel(const __grid_constant__ MarchParams p, int g_log2) {
@@ -1171,8 +1171,7 @@ __global__ void __launch_bounds__(128, 3)
             }
             float f[8] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f, 0.0f}, trans = 1.0f;
             if (lig < n) {
-                // what it waits on is the chain of loads: the widest groups of gates (50001
-                // rays, forward and reverse pass: 2190 us against 2263 one by one)
+                // what it waits on is the chain of loads: the widest groups of gates
                 sample_features<L, DT, AGG, false, false, GG>(p.g, my_u, p.opts.attn_mode, f, gate_smem + threadIdx.x,
                                                               blockDim.x);
                 trans = expf(-expf(f[0]) * my_delta);
@@ -1235,21 +1234,44 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
     constexpr int kBlocks = march_min_blocks<L, DT, AGG>();
     if constexpr (AGG == NGPRT_AGG_SEPARATE_V) {
         const int64_t rays = p.mode == 0 ? (int64_t)p.tiles_per_view * p.n_cams * 32 : p.n_rays;
-        // Several lanes a ray up to 2.4 times the threads that are resident at once: the
-        // lanes of a group share the long chain of a ray's samples, which pays even where
-        // the blocks take a second turn (hd, 57 k FP32 rays: 1387 us at two lanes, 1787 at
-        // one), and stops to when the GPU is full of rays anyway.  FP16 tables from four
-        // lanes on (57 k rays: 1203 us at two, 983 at one).  Stacks of up to 8 levels have
-        // shorter chains: from four lanes on, up to 1.8 times (8 levels, FP32: 18 k rays
-        // 390 us at four lanes, 575 at two or one; 36 k 760, 735 and 707; 68 k BF16 731 us
-        // at two, 508 at one).
+        // Several lanes a ray: the lanes of a group share the long chain of a ray's samples,
+        // which pays even where the blocks take a second turn, and stops to when the GPU is
+        // full of rays anyway.  In tenths of the threads that are resident at once, up to
+        // how many 2^g lanes are taken (us; "one" is a ray per lane):
+        //  - 16 and 32 lanes 1.2: samples past a ray's end cost as much as the others (hd,
+        //    4096 FP32 rays of 13 samples: 32 lanes 143, 16 85, one 230; of 20 samples 326
+        //    and 325; FP16 98, 47 and 195).
+        //  - 16 levels, 4 and 8 lanes 2.4 (hd, image of 14400: 8 lanes 575, 4 631, one 1850).
+        //  - 16 levels, 2 lanes 2.4 for images, 2.0 for lists, whose neighbours share less
+        //    (57 k pixels of an image 1387 against 1787; random ones 65 k 2334 against 1889);
+        //    FP16 tables never (57 k: 1203 against 983).
+        //  - up to 8 levels the chains are shorter: never 2 lanes (8 levels, 68 k BF16 rays
+        //    731 against 508); 8 lanes 1.6, 4 lanes 1.8 for FP32 and 1.2 for 16-bit tables (8
+        //    levels: 20 k free FP32 rays 358 at 4 lanes, 624 at one; FP16, 25 k pixels 573
+        //    and 460; 16 k 356 at 4, 378 at 8; image of 14400 286 at 8, 343 at 4).
+        //  - 2 to 4 levels of a contracted scene, where the walk through empty space, which
+        //    every lane of a group takes, outweighs the samples: from 8 lanes on (4 levels,
+        //    16 k rays 680 at 4 lanes, 513 at one; 8192 421 at 8).
+        //  - bounded scenes have little empty space to walk: 1.8 from 4 lanes on (128 x 128
+        //    view of the small scene 160 at 4 lanes, 283 at one); so do 4 and 8 lanes of a
+        //    single 16-bit level, whose march alone is slow (image of 30000 585 and 1632).
+        // Where every ray ends at its first sample the group's other samples are in vain,
+        // and up to some 60 k such rays take longer than one by one (4096: 81 against 42).
         constexpr bool kShort = L <= 8;
         static int room_cache[16] = {0};
         if (!room_cache[dev]) room_cache[dev] = resident_blocks(march_group_kernel<L, DT, AGG>, shm);
         const int64_t room = (int64_t)room_cache[dev] * 128;
-        int g = 0;
-                while (g < 5 && (rays << (g + 1)) * 5 <= room * (kShort ? 9 : 12)) ++g;
-        if (g > (kShort || DT == NGPRT_F16 ? 1 : 0) && !p.fb_a_hat && !lattice(p)) {
+        const auto most = [&](int g) {
+            if (!kShort) return g == 1 ? (DT == NGPRT_F16 ? 0 : p.mode == 0 ? 24 : 20) : g < 4 ? 24 : 12;
+            if (g == 1) return 0;
+            if (p.g.bounded) return 18;
+            if (g > 3) return 12;
+            if (L == 1 && DT != NGPRT_F32) return 18;
+            return g == 3 ? 16 : L <= 4 ? 0 : DT == NGPRT_F32 ? 18 : 12;
+        };
+        int g = 5;
+        while (g > 0 && (rays << g) * 10 > room * most(g)) --g;
+        if (g > 0 && !p.fb_a_hat && !lattice(p)) {
             const unsigned blocks = (unsigned)(((rays << g) + 127) / 128);
             march_group_kernel<L, DT, AGG><<<blocks, 128, shm, st>>>(p, g);
             return;

@@ -6,6 +6,7 @@ import pytest
 
 torch = pytest.importorskip("torch")
 
+from paper_2407_10482_gb300 import scenes as S
 from test_gpu_records import _close, _render_gradients, _setup
 
 pytestmark = pytest.mark.gpu
@@ -101,3 +102,33 @@ def test_pixel_lists_in_tile_order(L):
 @pytest.mark.parametrize("pixels", [True, False])
 def test_more_rays_than_one_pass_of_records(pixels):
     _render_gradients(1, (1 << 18) + 4129, pixels)
+
+
+def _contracted(L, dtype):
+    """A contracted scene of L levels with tables small enough to draw quickly."""
+    from paper_2407_10482_gb300 import ngprt as ng
+    cfg = S.hd_config(L=L, N=S.level_resolutions(16, 1024, L), T_log2=14, R_O=64, n_occ_levels=4, W=643, H=517)
+    sc = S.make_scene(cfg)
+    dt = getattr(ng, dtype)
+    ds = ng.DeviceScene(cfg, sc.tables, sc.coarse, sc.mlp_w, table_dtype=dt, mlp_dtype=ng.F32 if dt == ng.F32 else ng.F16)
+    docc = ng.DeviceOcc(sc.occ, cfg.R_O, cfg.n_occ_levels)
+    return ng, cfg, ds, docc
+
+
+@pytest.mark.parametrize("L", [2, 8, 16])
+@pytest.mark.parametrize("dtype", ["F32", "F16", "BF16"])
+def test_batches_of_every_size_render_the_rays_of_a_full_one(L, dtype):
+    """Free rays in batches that take 32, 16, 8, 4, 2 and 1 lanes a ray and each block count
+    of the march, against the same rays in a batch that fills the GPU.  Decisions are equal;
+    the groups contract w = T (1 - t) into its sum, one rounding (2^-24) a sample, of at most
+    100 samples here."""
+    ng, cfg, ds, docc = _contracted(L, dtype)
+    rend = ng.Renderer(ds, docc)
+    o, d = (torch.as_tensor(x).cuda() for x in S.random_rays(330011, 4, False))
+    opts = S.default_options(cfg)
+    full = rend.render(opts, rays_o=o, rays_d=d, stats=True, state=True)
+    assert int(full["stats"][:, 1].max()) <= 100
+    for n in (1, 2000, 4097, 8191, 13001, 25000, 55001, 90000, 110003, 140001, 180000):
+        part = rend.render(opts, rays_o=o[:n].contiguous(), rays_d=d[:n].contiguous(), stats=True, state=True)
+        assert torch.equal(part["stats"], full["stats"][:n])
+        torch.testing.assert_close(part["state"], full["state"][:n], rtol=6e-6, atol=6e-6)
