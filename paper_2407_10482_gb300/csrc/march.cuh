@@ -340,11 +340,11 @@ __device__ __forceinline__ void sample_features(const Grid& g, const float u[3],
     // level) and each level's gated sum is taken in mixed precision (FP16 factors,
     // FP32 sum), without converting the level's features
     constexpr bool kHalfGates = DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V && !kKeep;
-    constexpr bool kFly = (kRec || fly_gates<L, DT, AGG>()) && !kKeep;
+    constexpr bool kFly = (kRec || (G > 0 && fly_gates<L, DT, AGG>())) && !kKeep;
     constexpr int NF = kFly ? kNFeat : NC;  // channels taken from the coarse rows up front
     // the gates of the levels to come, the next level's first
-    [[maybe_unused]] float og[G], bg[G];
-    [[maybe_unused]] __half2 hg[G], ccw[4];
+    [[maybe_unused]] float og[G > 0 ? G : 1], bg[G > 0 ? G : 1];
+    [[maybe_unused]] __half2 hg[G > 0 ? G : 1], ccw[4];
     uint32_t ufx[3] = {0u, 0u, 0u};
     if constexpr (DT != NGPRT_F32) {
 #pragma unroll
@@ -954,8 +954,9 @@ __device__ __forceinline__ int64_t next_tile(const MarchParams& p) {
     return t < (unsigned long long)tiles ? (int64_t)t : -1;
 }
 
-// Forward sampler: features (Eq. 6-8), alpha compositing (Eq. 2, Eq. 5).
-template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V>
+// Forward sampler: features (Eq. 6-8; G as sample_features), alpha compositing (Eq. 2,
+// Eq. 5).
+template <int L, int DT, int AGG = NGPRT_AGG_SEPARATE_V, int G = gate_group<L, DT>()>
 struct ForwardSampler {
     const Grid& g;
     int attn_mode;
@@ -1001,7 +1002,7 @@ struct ForwardSampler {
     }
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
         float f[8];
-        sample_features<L, DT, AGG>(g, u, attn_mode, f, gates, blockDim.x);
+        sample_features<L, DT, AGG, false, false, G>(g, u, attn_mode, f, gates, blockDim.x);
         return composite(f, t, delta);
     }
 };
@@ -1076,6 +1077,14 @@ constexpr int march_min_blocks() {
 
 constexpr int kWideBlocks = 5;
 
+// Gate group of the march kernel of kBlocks blocks per SM.  FP32 stacks of more than 8 levels
+// hold all gates where the registers are there (hd, 90000 random pixels 2054 us against
+// 2197 one by one; images of 85000 and 120000 the same within 1.5%).
+template <int L, int DT, int kBlocks>
+constexpr int march_gates() {
+    return kBlocks == kWideBlocks && DT == NGPRT_F32 && L > 8 ? 0 : gate_group<L, DT>();
+}
+
 // kBlocks: blocks per SM (march_min_blocks, or kWideBlocks for small batches).
 template <int L, int DT, int AGG, int kBlocks>
 __global__ void __launch_bounds__(128, kBlocks) march_kernel(const __grid_constant__ MarchParams p) {
@@ -1093,7 +1102,7 @@ __global__ void __launch_bounds__(128, kBlocks) march_kernel(const __grid_consta
             const bool was_full = lo == -INFINITY && hi == INFINITY;
             if (was_full || !(p.fb_a_hat[ray] - s[7] > p.fb_thr)) return;
         }
-        ForwardSampler<L, DT, AGG> smp(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x);
+        ForwardSampler<L, DT, AGG, march_gates<L, DT, kBlocks>()> smp(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x);
         int n_march = 0, n_samp = 0;
         if (hit) march_loop<decltype(snap)::value>(p, ry, smp, n_march, n_samp);
         reinterpret_cast<float4*>(s)[0] = make_float4(smp.Cd[0], smp.Cd[1], smp.Cd[2], smp.F[0]);
@@ -1277,15 +1286,25 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
             return;
         }
         // Batches that do not fill the SMs with kBlocks blocks gain nothing from them, and
-        // lose to the spills that buy them: 5 blocks (96 registers) up to 1.5 times their
-        // resident threads.  hd, 77 k rays: FP32 1807 us against 1924, FP16 1002 against
-        // 1139, BF16 1277 against 1387; 120 k: 2074 and 2065, 1141 and 1211, 1471 and 1472;
-        // 224 k: 2578 and 2558, 1487 and 1495, 1932 and 1866.
-        static int wide_cache[16] = {0};
-        if (!wide_cache[dev]) wide_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kWideBlocks>, shm);
-        if (!p.fb_a_hat && rays * 2 <= (int64_t)wide_cache[dev] * 128 * 3) {
+        // lose to the spills that buy them.  Images take 5 blocks (96 registers) up to 1.5
+        // times their resident threads: their warps differ in length and fill a second turn
+        // (hd, 77 k rays: FP32 1807 us against 1924, FP16 1002 against 1139, BF16 1277 against
+        // 1387; 120 k: 2074 and 2065, 1141 and 1211, 1471 and 1472; 224 k: 2578 and 2558,
+        // 1487 and 1495, 1932 and 1866).  Lists take them where they need no turn more than
+        // kBlocks blocks would: a warp of unrelated rays is as long as its longest, so that
+        // every turn is whole (random pixels, FP16, 16 levels: 100 k 1992 us in two turns of 5
+        // blocks, 1499 in one of 8; FP32, 140 k, two turns either way: 3742 and 4224).
+        constexpr size_t wshm = march_gates<L, DT, kWideBlocks>() > 0
+                                    ? (size_t)gate_floats<L, DT, AGG>() * 128 * sizeof(float)
+                                    : (size_t)2 * L * 128 * sizeof(float);
+        static int wide_cache[16] = {0}, full_cache[16] = {0};
+        if (!wide_cache[dev]) wide_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kWideBlocks>, wshm);
+        if (!full_cache[dev]) full_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kBlocks>, shm);
+        const int64_t wide = (int64_t)wide_cache[dev] * 128, full = (int64_t)full_cache[dev] * 128;
+        const bool few = p.mode == 0 ? rays * 2 <= wide * 3 : rays <= wide || (rays > full && rays <= 2 * wide);
+        if (few && !p.fb_a_hat) {
             if (p.tile_counter && grid.x > (unsigned)wide_cache[dev]) grid.x = (unsigned)wide_cache[dev];
-            march_kernel<L, DT, AGG, kWideBlocks><<<grid, 128, shm, st>>>(p);
+            march_kernel<L, DT, AGG, kWideBlocks><<<grid, 128, wshm, st>>>(p);
             return;
         }
     }
