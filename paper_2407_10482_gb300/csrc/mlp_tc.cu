@@ -256,8 +256,11 @@ __global__ void __launch_bounds__(128) mlp_tc_kernel(const __grid_constant__ Mlp
 
 // CTAs per SM: each runs its tile's load, two or three MMAs and epilogues as one chain, so
 // several hide each other's latencies.  Four take all 512 TMEM columns of an SM and 4 x 39
-// KB of shared memory (1920 x 1080 FP16 frame: 6.69 ms at 2, 6.65 at 3, 6.64 at 4).
-constexpr int kCtasPerSm = 4;
+// KB of shared memory (1920 x 1080 FP16 frame: 6.69 ms at 2, 6.65 at 3, 6.64 at 4; 2^20
+// rays, the MLP alone, 56 us at 2 and 45 at 4).  Below some ten tiles an SM the CTAs' setup
+// (weights, TMEM) outweighs that: two (90000 rays 12.5 us at 2 and 16.5 at 4; 200000 18.6
+// and 18.9).
+constexpr int kCtasPerSm = 4, kFewCtasPerSm = 2, kManyTiles = 152 * 10;
 
 template <int WIDTH, int LAYERS>
 void launch_tc(const MlpTcParams& p, cudaStream_t st) {
@@ -266,7 +269,8 @@ void launch_tc(const MlpTcParams& p, cudaStream_t st) {
     if (shm > 48 * 1024)
         cudaFuncSetAttribute(mlp_tc_kernel<WIDTH, LAYERS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)shm);
     const int64_t tiles = (p.n + kTile - 1) / kTile;
-    const int64_t grid = tiles < 152 * kCtasPerSm ? tiles : 152 * kCtasPerSm;
+    const int64_t most = 152 * (tiles >= kManyTiles ? kCtasPerSm : kFewCtasPerSm);
+    const int64_t grid = tiles < most ? tiles : most;
     mlp_tc_kernel<WIDTH, LAYERS><<<(unsigned)grid, 128, shm, st>>>(p);
 }
 

@@ -250,9 +250,13 @@ bool mlp_supports(int width, int layers) {
 
 template <int WIDTH, int LAYERS>
 void launch_mlp_w(const MlpParams& p, cudaStream_t st) {
-    // two rays per thread once the blocks of 256 rays still give every SM its resident
-    // ones (152 SMs x 2 blocks); below that more, smaller blocks finish earlier
-    if (p.n >= 152 * 2 * 256) mlp_f32_kernel<WIDTH, LAYERS, 2><<<(unsigned)((p.n + 255) / 256), 128, 0, st>>>(p);
+    // Two rays per thread once the blocks of 256 rays still give every SM its resident ones
+    // (152 SMs x 2 blocks); below that more, smaller blocks finish earlier.  64 wide, where a
+    // turn of them is all that an SM holds, from 8 turns on: a half-empty last one costs more
+    // than the 6% that they save (3 layers: 90000 rays 43.9 us with one ray and 51.4 with two,
+    // 200000 74.8 and 76.0, 2^20 361 and 340; 16 wide: 200000 10.5 and 9.5, 2^20 35 and 29).
+    constexpr int64_t kTurn = 152 * 2 * 256;
+    if (p.n >= kTurn * (WIDTH >= 64 ? 8 : 1)) mlp_f32_kernel<WIDTH, LAYERS, 2><<<(unsigned)((p.n + 255) / 256), 128, 0, st>>>(p);
     else mlp_f32_kernel<WIDTH, LAYERS, 1><<<(unsigned)((p.n + 127) / 128), 128, 0, st>>>(p);
 }
 
