@@ -137,7 +137,8 @@ __global__ void __launch_bounds__(128, !kList && L == 8 ? 5 : 0) distortion_back
 // set), or NULL.
 template <int L>
 void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, float* g_plane, cudaStream_t st) {
-    const size_t shm = (size_t)gate_floats<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V>() * 128 * sizeof(float);
+    const size_t shm =
+        (size_t)(backward ? gate_floats<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V>() : 2 * L) * 128 * sizeof(float);
     if (!backward) {
         if (p.m.plane) {
             static int cache[16] = {0};

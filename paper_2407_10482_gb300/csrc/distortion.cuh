@@ -61,10 +61,11 @@ __device__ __forceinline__ void distortion_ray(const DistParams& p, const Weight
 // Shared gates of 16 levels at 3 blocks per SM (168 registers): left alone the compiler takes
 // 96 and spills (16384 rays 667 us against 568).
 template <int L, int AGG>
-__global__ void __launch_bounds__(128, L == 16 && AGG == NGPRT_AGG_SHARED_V ? 3 : 0) distortion_kernel(const __grid_constant__ DistParams p) {
+__global__ void __launch_bounds__(128, L == 16 && AGG == NGPRT_AGG_SHARED_V ? 3 : 0)
+    distortion_kernel(const __grid_constant__ DistParams p) {
     extern __shared__ float gate_smem[];
-    distortion_ray<true>(p, ForwardSampler<L, NGPRT_F32, AGG>(p.m.g, p.m.opts.attn_mode, p.m.opts.t_term,
-                                                        gate_smem + threadIdx.x));
+    using Weights = ForwardSampler<L, NGPRT_F32, AGG, kGatesUpFront>;
+    distortion_ray<true>(p, Weights(p.m.g, p.m.opts.attn_mode, p.m.opts.t_term, gate_smem + threadIdx.x));
 }
 
 // The same from the density channel alone (p.m.plane), tiles handed out at run time.

@@ -182,6 +182,16 @@ template <int L, int DT>
 constexpr int gate_group() {
     return DT == NGPRT_F32 || L % 2 != 0 ? 1 : L % 4 == 0 ? 4 : 2;
 }
+// The group of the other passes that interpolate all channels (regulariser, visibility marks,
+// density grid, proposal targets): all gates up front.  They run one ray or voxel a lane
+// through the general march, where the loads of a group come on top of every level's chain
+// (hd, us up front and by groups: regulariser of 16384 random pixels 1207 and 2221, marks
+// BF16 802 and 1216, density at 32^3 FP32 32 and 39, FP16 19 and 27).
+constexpr int kGatesUpFront = 0;
+// Blocks per SM of those marches: FP32 stacks of more than 8 levels need the registers of 5
+// (proposal targets of 16384 random pixels 1235 us at 5 and 1379 at 7).
+template <int L, int DT, int AGG>
+constexpr int general_min_blocks();
 
 // G consecutive 32-bit words (aligned to all of them).
 template <int G>
@@ -718,10 +728,10 @@ __device__ __forceinline__ float sample_density(const Grid& g, const float* __re
     return f0;
 }
 
-// Shared-memory floats per thread that sample_features parks its gates in.
-template <int L, int DT, int AGG>
+// Shared-memory floats per thread that sample_features parks its gates in (G as there).
+template <int L, int DT, int AGG, int G = gate_group<L, DT>()>
 __host__ __device__ constexpr int gate_floats() {
-    if (AGG == NGPRT_AGG_SUM || AGG == NGPRT_AGG_MLP || fly_gates<L, DT, AGG>()) return 0;
+    if (AGG == NGPRT_AGG_SUM || AGG == NGPRT_AGG_MLP || (G > 0 && fly_gates<L, DT, AGG>())) return 0;
     return DT == NGPRT_F16 && AGG == NGPRT_AGG_SEPARATE_V ? L : 2 * L;
 }
 
@@ -1077,6 +1087,11 @@ constexpr int march_min_blocks() {
 
 constexpr int kWideBlocks = 5;
 
+template <int L, int DT, int AGG>
+constexpr int general_min_blocks() {
+    return DT == NGPRT_F32 && AGG == NGPRT_AGG_SEPARATE_V && L > 8 ? kWideBlocks : march_min_blocks<L, DT, AGG>();
+}
+
 // Gate group of the march kernel of kBlocks blocks per SM.  FP32 stacks of more than 8 levels
 // hold all gates where the registers are there (hd, 90000 random pixels 2054 us against
 // 2197 one by one; images of 85000 and 120000 the same within 1.5%).
@@ -1294,9 +1309,8 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
         // kBlocks blocks would: a warp of unrelated rays is as long as its longest, so that
         // every turn is whole (random pixels, FP16, 16 levels: 100 k 1992 us in two turns of 5
         // blocks, 1499 in one of 8; FP32, 140 k, two turns either way: 3742 and 4224).
-        constexpr size_t wshm = march_gates<L, DT, kWideBlocks>() > 0
-                                    ? (size_t)gate_floats<L, DT, AGG>() * 128 * sizeof(float)
-                                    : (size_t)2 * L * 128 * sizeof(float);
+        constexpr size_t wshm =
+            (size_t)gate_floats<L, DT, AGG, march_gates<L, DT, kWideBlocks>()>() * 128 * sizeof(float);
         static int wide_cache[16] = {0}, full_cache[16] = {0};
         if (!wide_cache[dev]) wide_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kWideBlocks>, wshm);
         if (!full_cache[dev]) full_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kBlocks>, shm);

@@ -31,7 +31,8 @@ __global__ void __launch_bounds__(128) density_occ_kernel(const __grid_constant_
                         fmul(fadd((float)k, 0.5f), inv)};
     float f[8];
     if constexpr (kPlane) f[0] = sample_density<L>(p.g, p.plane, u, p.attn_mode);
-    else sample_features<L, DT, AGG>(p.g, u, p.attn_mode, f, gate_smem + threadIdx.x, blockDim.x);
+    else sample_features<L, DT, AGG, false, false, kGatesUpFront>(p.g, u, p.attn_mode, f, gate_smem + threadIdx.x,
+                                                                  blockDim.x);
     const float sg = expf(f[0]);
     p.occ[v] = sg > p.sigma_thr ? 1 : 0;
     if (p.sigma) p.sigma[v] = sg;
@@ -57,15 +58,16 @@ struct VisibilitySampler {
 };
 
 template <int L, int DT, int AGG>
-__global__ void __launch_bounds__(128, march_min_blocks<L, DT, AGG>())
+__global__ void __launch_bounds__(128, general_min_blocks<L, DT, AGG>())
     visibility_kernel(const __grid_constant__ MarchParams p, float w_thr, int32_t R, uint8_t* vis) {
     int64_t ray;
     Ray ry;
     bool hit;
     extern __shared__ float gate_smem[];
     if (!ray_setup(p, ray, ry, hit)) return;
-    VisibilitySampler<ForwardSampler<L, DT, AGG>> smp{
-        ForwardSampler<L, DT, AGG>(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x), w_thr, R, vis};
+    using Weights = ForwardSampler<L, DT, AGG, kGatesUpFront>;
+    VisibilitySampler<Weights> smp{Weights(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x), w_thr, R,
+                                   vis};
     int n_march = 0, n_samp = 0;
     if (hit) march_loop(p, ry, smp, n_march, n_samp);
 }
@@ -98,8 +100,9 @@ void launch_density(int dt, const DensityOccParams& p, cudaStream_t st) {
             return;
         }
     }
-    const size_t shm = 128 * sizeof(float), f32 = gate_floats<L, NGPRT_F32, AGG>() * shm,
-                 f16 = gate_floats<L, NGPRT_F16, AGG>() * shm, bf16 = gate_floats<L, NGPRT_BF16, AGG>() * shm;
+    const size_t shm = 128 * sizeof(float), f32 = gate_floats<L, NGPRT_F32, AGG, kGatesUpFront>() * shm,
+                 f16 = gate_floats<L, NGPRT_F16, AGG, kGatesUpFront>() * shm,
+                 bf16 = gate_floats<L, NGPRT_BF16, AGG, kGatesUpFront>() * shm;
     if (dt == NGPRT_F32) density_occ_kernel<L, NGPRT_F32, AGG><<<blocks, 128, f32, st>>>(p);
     else if (dt == NGPRT_F16) density_occ_kernel<L, NGPRT_F16, AGG><<<blocks, 128, f16, st>>>(p);
     else density_occ_kernel<L, NGPRT_BF16, AGG><<<blocks, 128, bf16, st>>>(p);
@@ -114,8 +117,9 @@ void launch_visibility(int dt, const MarchParams& p, dim3 grid, float w_thr, int
             return;
         }
     }
-    const size_t shm = 128 * sizeof(float), f32 = gate_floats<L, NGPRT_F32, AGG>() * shm,
-                 f16 = gate_floats<L, NGPRT_F16, AGG>() * shm, bf16 = gate_floats<L, NGPRT_BF16, AGG>() * shm;
+    const size_t shm = 128 * sizeof(float), f32 = gate_floats<L, NGPRT_F32, AGG, kGatesUpFront>() * shm,
+                 f16 = gate_floats<L, NGPRT_F16, AGG, kGatesUpFront>() * shm,
+                 bf16 = gate_floats<L, NGPRT_BF16, AGG, kGatesUpFront>() * shm;
     if (dt == NGPRT_F32) visibility_kernel<L, NGPRT_F32, AGG><<<grid, 128, f32, st>>>(p, w_thr, R, vis);
     else if (dt == NGPRT_F16) visibility_kernel<L, NGPRT_F16, AGG><<<grid, 128, f16, st>>>(p, w_thr, R, vis);
     else visibility_kernel<L, NGPRT_BF16, AGG><<<grid, 128, bf16, st>>>(p, w_thr, R, vis);

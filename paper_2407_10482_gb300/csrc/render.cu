@@ -17,9 +17,9 @@ namespace ngprt {
 // render, the position of the first sample whose cumulative weight exceeds
 // 0.005 A, the end (t + delta) of the first sample whose cumulative weight reaches
 // 0.995 A, and A.  The samples are the forward's (same march, same compositing).
-template <int L, int DT>
+template <class Weights>
 struct TargetSampler {
-    ForwardSampler<L, DT> fw;
+    Weights fw;
     float A_final, t_near, t_far;
     bool got_near, got_far;
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
@@ -38,16 +38,17 @@ struct TargetSampler {
 };
 
 template <int L, int DT>
-__global__ void __launch_bounds__(128, march_min_blocks<L, DT>()) targets_kernel(const __grid_constant__ MarchParams p,
-                                                                                float* targets) {
+__global__ void __launch_bounds__(128, general_min_blocks<L, DT, NGPRT_AGG_SEPARATE_V>())
+    targets_kernel(const __grid_constant__ MarchParams p, float* targets) {
     extern __shared__ float gate_smem[];
     int64_t ray;
     Ray ry;
     bool hit;
     if (!ray_setup(p, ray, ry, hit)) return;
     const float A = p.state[ray * NGPRT_STATE_FLOATS + 7];
-    TargetSampler<L, DT> smp{ForwardSampler<L, DT>(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x), A,
-                             0.0f, 0.0f, false, false};
+    using Weights = ForwardSampler<L, DT, NGPRT_AGG_SEPARATE_V, kGatesUpFront>;
+    TargetSampler<Weights> smp{Weights(p.g, p.opts.attn_mode, p.opts.t_term, gate_smem + threadIdx.x), A, 0.0f, 0.0f,
+                               false, false};
     int n_march = 0, n_samp = 0;
     if (hit) march_loop(p, ry, smp, n_march, n_samp);
     if (n_samp == 0) smp.t_far = 0.0f;

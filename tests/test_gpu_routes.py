@@ -132,3 +132,19 @@ def test_batches_of_every_size_render_the_rays_of_a_full_one(L, dtype):
         part = rend.render(opts, rays_o=o[:n].contiguous(), rays_d=d[:n].contiguous(), stats=True, state=True)
         assert torch.equal(part["stats"], full["stats"][:n])
         torch.testing.assert_close(part["state"], full["state"][:n], rtol=6e-6, atol=6e-6)
+
+
+@pytest.mark.parametrize("L", [2, 8, 16])
+@pytest.mark.parametrize("dtype,rtol", [("F16", 0.05), ("BF16", 1e-3)])
+def test_density_grid_of_16_bit_tables(L, dtype, rtol):
+    """Against FP32 tables of the rounded values.  BF16 differs by the rounding of FP32 sums
+    and of the fixed-point cells; FP16 by its half2 sums: 8 roundings of 2^-11 of a raw
+    density of about 4, 0.016, and as much for the levels together, in the exponent."""
+    ng, cfg, ds, docc = _contracted(L, dtype)
+    ds32 = ng.DeviceScene(cfg, ds.tables.float(), ds.coarse.float(), ds.mlp_w.float())
+    ro, R = ng.render_opts(S.default_options(cfg)), 32
+    occ = torch.empty(R ** 3, dtype=torch.uint8, device="cuda")
+    sigma = [torch.empty(R ** 3, device="cuda") for _ in range(2)]
+    for scene, out in zip((ds, ds32), sigma):
+        ng.ngprt_occupancy_from_density(scene.struct, ro, R, 20.0, occ, out)
+    torch.testing.assert_close(sigma[0], sigma[1], rtol=rtol, atol=0)
