@@ -62,9 +62,14 @@ constexpr int64_t kRecordMinRays = 4096;   // fewer rays take the one-kernel for
 // add to the same rows at the same time and wait for one another (us without records, in
 // tile order and in the given order: 2 levels, 16384 random pixels 503, 806 and 555; 16
 // levels, 32768 2890, 2122 and 1963); above, their gathers meet in L1 (16 levels, 2^17
-// 10622, 4559 and 5301).  The regulariser's records never are: 16 levels, 2^16 1892 and
-// 1681; 2 levels, 16384 747 and 473, without records 516.
+// 10622, 4559 and 5301).  Tables of fewer than 2^16 rows, all of them hot whatever the
+// order, from half as many on (bounded 4 levels of 2^12 rows, 50001 pixels on a full grid
+// 1171, 956 and 1279).  The regulariser's records never are: 16 levels, 2^16 1892 and 1681;
+// 2 levels, 16384 747 and 473, without records 516.
 constexpr int64_t kBinRays = 1 << 16;
+inline bool tile_order_pays(const MarchParams& m, int L) {
+    return m.n_rays >= (((int64_t)m.g.T_mask + 1) * L < 1 << 16 ? kBinRays / 2 : kBinRays);
+}
 // Pixel lists of 2 and 4 levels take the one-kernel form up to so many rays: it adds whole
 // rows of their coarse grid at a time, and its latency hides what records save (16384
 // pixels: 2 levels 503 us against 555, 4 levels 603 against 669, bounded 488 against 523;
@@ -530,7 +535,7 @@ inline RecLayout record_layout(int L, bool dist, int64_t n_rays) {
     a.max_chunks = (uint32_t)(want < room ? want : room);
     size_t at = 0;
     a.counters = at; at += 256;
-    a.order = !dist && n_rays >= kBinRays;
+    a.order = !dist && n_rays >= kBinRays / 2;
     a.perm = at; at += a.order ? up((size_t)n_rays * sizeof(int32_t)) : 0;
     a.bins = at; at += a.order ? up((size_t)kMaxBins * sizeof(uint32_t)) : 0;
     a.list = at; at += up((size_t)pass * sizeof(int2));
@@ -624,7 +629,7 @@ void launch_records(RecParams p, void* scratch, cudaStream_t st, Rest rest) {
     p.rec = reinterpret_cast<float*>(base + a.rec);
     p.max_chunks = a.max_chunks;
     p.perm = nullptr;
-    if (a.order)
+    if (a.order && tile_order_pays(p.m, L))
         p.perm = bin_rays(p.m, reinterpret_cast<uint32_t*>(base + a.bins), reinterpret_cast<int32_t*>(base + a.perm), st);
     static int cache1[16] = {0}, cache2[16] = {0}, cache3[16] = {0};
     const unsigned g1 = resident_grid(record_kernel<L, kDist>, cache1),

@@ -148,3 +148,32 @@ def test_density_grid_of_16_bit_tables(L, dtype, rtol):
     for scene, out in zip((ds, ds32), sigma):
         ng.ngprt_occupancy_from_density(scene.struct, ro, R, 20.0, occ, out)
     torch.testing.assert_close(sigma[0], sigma[1], rtol=rtol, atol=0)
+
+
+def test_small_tables_in_tile_order():
+    """Few table rows: the pixel-tile order from 2^15 rays on."""
+    from paper_2407_10482_gb300 import ngprt as ng
+    cfg = S.small_config(blob_std=(0.05, 0.15), W=160, H=96)
+    sc = S.make_scene(cfg)
+    ds = ng.DeviceScene(cfg, sc.tables, sc.coarse, sc.mlp_w)
+    docc = ng.DeviceOcc(sc.occ, cfg.R_O, cfg.n_occ_levels)
+    opts, n = S.default_options(cfg), (1 << 15) + 33
+    rays = dict(cams=S.orbit_cameras(cfg, 3, azimuth0=5.0), W=cfg.W, H=cfg.H,
+                pixel_ids=torch.as_tensor(S.random_pixels(n, 3, cfg.W, cfg.H, 2)).cuda())
+    rend = ng.Renderer(ds, docc)
+    out = rend.render(opts, state=True, **rays)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    d_rgb = torch.randn(n, 3, device="cuda", generator=gen)
+    cams, n_cams = ng.cameras_struct(rays["cams"], cfg.W, cfg.H)
+    ro = ng.render_opts(opts)
+    got = []
+    for need in (ng.ngprt_render_backward_scratch_bytes(ds.struct, ro, n),
+                 ng.ngprt_render_backward_workspace_bytes(ds.struct, ro, n)):
+        g = [torch.zeros_like(t) for t in (ds.tables, ds.coarse, ds.mlp_w)]
+        ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+        ng.ngprt_render_backward(ds.struct, docc.struct, cams, n_cams, rays["pixel_ids"], None, None, n, ro,
+                                 out["state"], d_rgb, None, None, *g, ws)
+        got.append(g)
+    for a, b in zip(*got):
+        _close(a, b)
