@@ -177,3 +177,115 @@ def test_small_tables_in_tile_order():
         got.append(g)
     for a, b in zip(*got):
         _close(a, b)
+
+
+@pytest.mark.parametrize("mode", ["tiles", "pixel_ids", "rays"])
+@pytest.mark.parametrize("dtype", ["F32", "F16", "BF16"])
+def test_run_time_tiles_of_batches_beyond_the_resident_warps(mode, dtype):
+    """More tiles than the GPU holds warps, so that warps take several from the counter:
+    bit for bit the static grid's states and counts."""
+    ng, cfg, ds, docc = _contracted(16, dtype)
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    ro = ng.render_opts(S.default_options(cfg))
+    cams, n_cams = ng.cameras_struct(S.orbit_cameras(cfg, 3, azimuth0=7.0, step_deg=120.0), cfg.W, cfg.H)
+    pix = o = d = None
+    n = sms * 64 * 32 + 18011
+    if mode == "tiles":
+        n = n_cams * cfg.W * cfg.H
+    elif mode == "pixel_ids":
+        pix = torch.as_tensor(S.random_pixels(n, 3, cfg.W, cfg.H, 5)).cuda()
+    else:
+        o, d = (torch.as_tensor(x).cuda() for x in S.random_rays(n, 9, False))
+        cams, n_cams = None, 0
+    assert (n + 31) // 32 > sms * 64
+    out = []
+    for ws_bytes in (0, ng.ngprt_render_workspace_bytes(ds.struct, n)):
+        state = torch.full((n, ng.STATE_FLOATS), float("nan"), device="cuda")
+        stats = torch.full((n, 2), -1, dtype=torch.int32, device="cuda")
+        ws = torch.empty(ws_bytes, dtype=torch.uint8, device="cuda") if ws_bytes else None
+        for _ in range(2):
+            ng.ngprt_render(ds.struct, docc.struct, cams, n_cams, pix, o, d, n, None, ro, None, ray_stats=stats,
+                            ray_state=state, workspace=ws)
+        out.append((state.view(torch.int32), stats))
+    assert bool((out[0][1] >= 0).all())
+    assert torch.equal(out[0][0], out[1][0]) and torch.equal(out[0][1], out[1][1])
+
+
+@pytest.mark.parametrize("attn_mode", [0, 1, 2])
+@pytest.mark.parametrize("L", [1, 4, 8, 16])
+def test_distortion_records_of_every_gate_mode(L, attn_mode):
+    for pixels in (True, False):
+        for a, b in zip(*_distortion_gradients(L, 4096 + 33, pixels, attn_mode=attn_mode)):
+            _close(a, b)
+
+
+def _whole_images(ng, ds, docc, cfg, views=2):
+    cams = S.orbit_cameras(cfg, views, azimuth0=5.0)
+    arr, n_cams = ng.cameras_struct(cams, cfg.W, cfg.H)
+    return views * cfg.W * cfg.H, dict(cams=cams, W=cfg.W, H=cfg.H), (arr, n_cams, None, None, None)
+
+
+@pytest.mark.parametrize("L", [1, 2, 8, 16])
+def test_whole_images_by_records(L):
+    """Camera images without a pixel list: render's and the regulariser's reverse passes."""
+    ng, ds, occ, opts, _, _ = _setup(L, 1, True)
+    n, rays, src = _whole_images(ng, ds, occ, ds.cfg)
+    ro, rend = ng.render_opts(opts), ng.Renderer(ds, occ)
+    out = rend.render(opts, state=True, **rays)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    d_rgb = torch.randn(n, 3, device="cuda", generator=gen)
+    got = []
+    for need in (ng.ngprt_render_backward_scratch_bytes(ds.struct, ro, n),
+                 ng.ngprt_render_backward_workspace_bytes(ds.struct, ro, n)):
+        g = [torch.zeros_like(t) for t in (ds.tables, ds.coarse, ds.mlp_w)]
+        ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+        ng.ngprt_render_backward(ds.struct, occ.struct, *src, n, ro, out["state"], d_rgb, None, None, *g, ws)
+        got.append(g)
+    for a, b in zip(*got):
+        _close(a, b)
+    state = torch.empty(n, 4, device="cuda")
+    ng.ngprt_distortion_loss(ds.struct, occ.struct, *src, n, ro, 1.0, state)
+    g = [[torch.zeros_like(t) for t in (ds.tables, ds.coarse)] for _ in range(2)]
+    ng.ngprt_distortion_backward(ds.struct, occ.struct, *src, n, ro, state, 1.0 / n, *g[0])
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert ng.lib().ngprt_distortion_backward(
+        C.byref(ds.struct), C.byref(occ.struct), src[0], src[1], None, None, None, n, C.byref(ro), _ptr(state),
+        C.c_float(1.0 / n), _ptr(g[1][0]), _ptr(g[1][1]), None, None, None, 0, st) == 0
+    for a, b in zip(*g):
+        _close(a, b)
+
+
+def test_calls_under_capture():
+    """A render of a small batch (kernels this process may not have used yet), its reverse
+    pass, the regulariser and the marks, captured at first use and replayed, against the
+    same calls outside."""
+    n = 4129
+    ng, ds, occ, opts, rays, src = _setup(3, n, True, t_term=0.01)
+    ro, rend = ng.render_opts(opts), ng.Renderer(ds, occ)
+    d_rgb = torch.ones(n, 3, device="cuda") / n
+    rend.workspace(n)
+
+    def calls():
+        out = rend.render(opts, state=True, **rays)
+        g = [torch.zeros_like(t) for t in (ds.tables, ds.coarse, ds.mlp_w)]
+        rend.backward(opts, out["state"], d_rgb, None, None, *g, **rays)
+        state = torch.empty(n, 4, device="cuda")
+        ng.ngprt_distortion_loss(ds.struct, occ.struct, *src, n, ro, 1.0, state)
+        gd = [torch.zeros_like(t) for t in (ds.tables, ds.coarse)]
+        ng.ngprt_distortion_backward(ds.struct, occ.struct, *src, n, ro, state, 1.0 / n, *gd)
+        vis = torch.zeros(32 ** 3, dtype=torch.uint8, device="cuda")
+        ng.ngprt_occupancy_visibility(ds.struct, occ.struct, *src, n, ro, 1e-3, 32, vis)
+        return [out["rgb"], out["state"], vis, state], g + gd
+
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        same, close = calls()
+    graph.replay()
+    torch.cuda.synchronize()
+    ref_same, ref_close = calls()
+    for a, b in zip(same, ref_same):
+        assert torch.equal(a, b)
+    for a, b in zip(close, ref_close):
+        _close(a, b)
