@@ -364,11 +364,12 @@ int32_t ngprt_shade(const ngprt_scene* scene, const float* ray_state, int64_t n_
  */
 size_t ngprt_render_backward_workspace_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
                                              int64_t n_rays);
-/* Bytes with which ngprt_render_backward is fastest (>= the workspace bytes; about 11 KB
- * a ray at L = 16, for at most 2^18 rays at a time): it then records the samples and sums
- * each ray's records per grid cell before adding to the gradients.  Any workspace from
- * ngprt_render_backward_workspace_bytes on is accepted; a smaller one than this takes
- * the form that adds every sample by itself. */
+/* Bytes with which ngprt_render_backward is fastest (>= the workspace bytes; 2.5 + 2 L KB
+ * a ray, at most 3 GB and the cotangents, for at most 2^18 rays at a time): it then records
+ * the samples and sums each ray's records per grid cell before adding to the gradients.
+ * Any workspace from ngprt_render_backward_workspace_bytes on is accepted; a smaller one
+ * than this takes the form that adds every sample by itself, and so do fewer than 4096 rays
+ * and lists of at most 2^15 pixels of 2 or 4 levels. */
 size_t ngprt_render_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts, int64_t n_rays);
 int32_t ngprt_render_backward(const ngprt_scene* scene, const ngprt_occ* occ, const ngprt_camera* cams,
                               int32_t n_cams, const int32_t* pixel_ids, const float* rays_o,

@@ -326,13 +326,14 @@ __device__ __forceinline__ void level_gates_h2(const Grid& g, uint32_t cb, uint3
 // Eq. 6-8 at unit-cube position u: f = f~ + Att(f^1..f^L; a), or one of the
 // aggregations of Table 3 (AGG, an ngprt_aggregation).  The coarse fetch
 // interpolates the coarse grid's channels (f~ and, for the spatially variant forms,
-// the attention logits); the 2L gates (sigmoid of the interpolated or constant
-// logits) are parked in shared memory, gates[k*stride], so that the level loop need
-// not be unrolled.  FP32 and BF16 tables interpolate in FP32; FP16 tables
-// interpolate in packed half2 FMAs with FP16 corner weights (FP16 products and
-// sums, one conversion per channel), the rest of the sample in FP32.  The 16-bit
-// forms take their cells with the conversion-free floor (grid_cell_fast).  The MLP form accumulates its 64 hidden
-// units level by level (W1 columns of level l against f^l), then applies W2.
+// the attention logits).  The gates (sigmoid of the interpolated or constant logits) are
+// either all found up front and parked in shared memory, gates[k*stride], so that the
+// level loop need not be unrolled, or for G levels at a time as they come (fly_gates;
+// G = 0: up front whatever it says).  FP32 and BF16 tables interpolate in FP32; FP16
+// tables interpolate in packed half2 FMAs with FP16 corner weights (FP16 products and
+// sums, one conversion per channel), the rest of the sample in FP32.  The 16-bit forms
+// take their cells from fixed-point coordinates (table_cell).  The MLP form accumulates
+// its 64 hidden units level by level (W1 columns of level l against f^l), then applies W2.
 // With kKeep (reverse pass), level l also leaves sigma^l and q^l = sum over the
 // colour channels of f^l times gq (the ray's colour cotangents) in the slots
 // gates[(2L + 2l) * stride] and gates[(2L + 2l + 1) * stride]; the MLP form leaves

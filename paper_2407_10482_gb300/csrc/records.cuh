@@ -38,7 +38,7 @@
 // that its gathers take from L2.
 //
 // The regulariser takes records up to kDistRecordRays rays: 2^16 camera pixels of the hd
-// scene, forward and reverse pass, 3.0 ms in place of 10.4; 8 levels 1.66 in place of 3.30.
+// scene, forward and reverse pass, 2.6 ms in place of 10.3; 8 levels 1.41 in place of 3.14.
 // Beyond, its reverse pass stays in one kernel.  The gradients of a row are many small
 // terms of both signs there, and what a float accumulator keeps of them depends on how
 // they are grouped: at 2^18 rays the one-kernel form is 4e-5 of the coarse gradient away
@@ -109,8 +109,8 @@ struct RecParams {
 
 template <int L, bool kDist>
 __global__ void __launch_bounds__(128, kDist ? 6 : 4) record_kernel(const __grid_constant__ RecParams p) {
-    // levels whose gates are interpolated at a time: 50001 rays of 8 levels, forward and
-    // reverse pass, 2105 us with 4 and 2190 one by one; 2^18 of 16 levels 12.65 and 12.58 ms
+    // levels whose gates are interpolated at a time: with 4, 50001 rays of 8 levels, forward
+    // and reverse pass, take 4% less than one by one; 2^18 of 16 levels 12.65 and 12.58 ms
     constexpr int RG = L % 4 == 0 ? 4 : L % 2 == 0 ? 2 : 1;
     constexpr int F = record_floats<L, kDist>();
     const int lane = threadIdx.x & 31;
@@ -213,7 +213,7 @@ __global__ void __launch_bounds__(128, kDist ? 6 : 4) record_kernel(const __grid
     }
 }
 
-// NL consecutive floats added at p (4-byte, 8-byte or 16-byte reductions by the row's
+// NV consecutive floats added at p (4-byte, 8-byte or 16-byte reductions by the row's
 // alignment kAlign, in floats).
 template <int NV, int kAlign>
 __device__ __forceinline__ void add_row(float* p, const float* v) {
