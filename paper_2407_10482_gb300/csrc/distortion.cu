@@ -254,7 +254,7 @@ static int32_t run_distortion(bool backward, const ngprt_scene* scene, const ngp
     // starts anywhere else (a view into a flat buffer) takes the one-kernel form's single
     // floats
     const bool wide = !backward || ((uintptr_t)g_coarse & 15) == 0;
-    if (workspace && (backward ? plane_serves(scene) : plane_pays(scene, n_rays)) && !lattice(p.m) && wide) {
+    if (workspace && (backward ? plane_pays_records(scene, n_rays) : plane_pays(scene, p.m)) && !lattice(p.m) && wide) {
         const int64_t entries = ngprt_table_entries(scene);
         const size_t plane = plane_layout(entries, backward ? 0 : n_rays, backward).bytes;
         const size_t rec = backward ? record_scratch_bytes(L, true, n_rays) : 0;
@@ -310,7 +310,7 @@ extern "C" size_t ngprt_distortion_backward_workspace_bytes(const ngprt_scene* s
 extern "C" size_t ngprt_distortion_backward_scratch_bytes(const ngprt_scene* scene, const ngprt_render_opts* opts,
                                                           int64_t n_rays) {
     const size_t b = ngprt_distortion_backward_workspace_bytes(scene, opts, n_rays);
-    if (n_rays < 0 || !plane_serves(scene)) return b;
+    if (n_rays < 0 || !plane_pays_records(scene, n_rays)) return b;
     const size_t rec = record_scratch_bytes(scene->L, true, n_rays);
     return rec ? plane_layout(ngprt_table_entries(scene), 0, true).bytes + rec : b;
 }

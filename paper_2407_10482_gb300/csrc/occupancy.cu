@@ -134,7 +134,7 @@ extern "C" int32_t ngprt_occupancy_visibility_ws(const ngprt_scene* scene, const
     }
     const bool built = scene->L <= 4 || scene->L == 8 || scene->L == 16;
     const size_t best = ngprt_density_scratch_bytes(scene, n_rays);
-    if (built && workspace && best && ws_bytes >= best && !lattice(p))
+    if (built && workspace && best && ws_bytes >= best && plane_pays(scene, p) && !lattice(p))
         density_scratch(p, ngprt_table_entries(scene), true, workspace, st);
     switch (scene->L) {
         case 1: launch_visibility<1, NGPRT_AGG_SEPARATE_V>(scene->table_dtype, p, grid, w_thr, R, vis, st); break;

@@ -75,8 +75,17 @@ inline bool tile_order_pays(const MarchParams& m, int L) {
 // pixels: 2 levels 503 us against 555, 4 levels 603 against 669, bounded 488 against 523;
 // 65536: 1266 against 863).
 constexpr int64_t kFewLevelRays = 1 << 15;
+//
+// A coarse grid as fine as the steps (the paper shape's 512^3) leaves the coarse rows no run
+// of samples to sum: there records start above 2^15 rays whatever their source, and with up
+// to 2 levels they serve pixel lists above 2^17 alone (paper shape, ms without records and
+// with: 4 levels, 16384 free rays 0.99 and 1.31, 65536 4.08 and 3.53; 2 levels, 2^18 free
+// rays 9.0 and 10.7, pixels 6.2 and 5.7, 65536 pixels 2.05 and 2.41).
 inline bool records_pay(int L, const MarchParams& m) {
-    return m.mode != 1 || (L != 2 && L != 4) || m.n_rays > kFewLevelRays;
+    const float cell = (m.g.bounded ? 2.0f : 4.0f) / (float)(m.g.R_C - 1);
+    const bool fine = cell < 4.0f * m.opts.step_base * m.opts.step_gamma;
+    if (fine && L <= 2) return m.mode == 1 && m.n_rays > 4 * kFewLevelRays;
+    return (!fine && (m.mode != 1 || (L != 2 && L != 4))) || m.n_rays > kFewLevelRays;
 }
 constexpr int64_t kDistRecordRays = 1 << 16;  // more rays of the regulariser take the one-kernel form
 constexpr int kMaxBins = 1 << 16;
@@ -585,15 +594,30 @@ inline bool plane_serves(const ngprt_scene* s) {
 }
 
 // Whether the plane's copy (hd, 6.1 M rows: 45 us; 42 M rows: 250 us) pays for a forward
-// pass over rays: from 4096 rays on, and a ray for every 2000 rows, for stacks of up to 4
-// levels, whose samples gain less, for every 140.  us without and with the plane,
+// pass over rays: from 4096 rays on, and a ray for every 2000 rows, for shorter stacks, whose
+// samples gain less, for every 700 (8 levels) or 140.  us without and with the plane,
 // visibility pass: hd, 1 ray 97 and 152, 1000 random pixels 1072 and 1038, 4096 1323 and
 // 889; 42 M rows, 1 ray 97 and 352, 6912 pixels of an image 1183 and 1332, 65536 1668 and
-// 1399; 2 levels, 1 M rows, 4096 free rays 239 and 250, 65536 344 and 327.  (Where every ray
-// ends after some 14 samples the copy does not pay back at 4096 rays: 174 and 219.)
+// 1399; 8 levels, 52 M rows, 32768 pixels 805 and 1089; 4 levels, 17 M rows, 16384 1005 and
+// 1253, 2^18 3436 and 1724.  (Where every ray ends after some 14 samples the copy does not
+// pay back at 4096 rays: 174 and 219.)  Up to 3 levels of 2^20 rows or more gain by the
+// pixel-tile order alone (8 M rows, 2^18 pixels 2892 and 1378, free rays 3965 and 5053).
 inline bool plane_pays(const ngprt_scene* s, int64_t n_rays) {
-    return plane_serves(s) && n_rays >= kRecordMinRays &&
-           n_rays >= ngprt_table_entries(s) / (s->L <= 4 ? 140 : 2000);
+    if (!plane_serves(s)) return false;
+    const int64_t rows = ngprt_table_entries(s);
+    return n_rays >= kRecordMinRays && n_rays >= rows / (s->L <= 2 ? 67 : s->L <= 4 ? 140 : s->L <= 8 ? 700 : 2000);
+}
+inline bool plane_pays(const ngprt_scene* s, const MarchParams& m) {
+    return plane_pays(s, m.n_rays) && (s->L > 3 || m.mode == 1 || ngprt_table_entries(s) < 1 << 20);
+}
+
+// The same for the regulariser's records, which take a second plane, of the gradient: us
+// without and with, 4 levels, 17 M rows, 16384 free rays 1097 and 1401, 65536 5587 and 3457;
+// 16 levels, 80 M rows, 4096 pixels 1777 and 1710, 16384 2338 and 2000.
+inline bool plane_pays_records(const ngprt_scene* s, int64_t n_rays) {
+    if (!plane_serves(s)) return false;
+    const int64_t rows = ngprt_table_entries(s);
+    return n_rays >= rows / (s->L <= 3 ? 200 : s->L <= 4 ? 400 : 16000);
 }
 
 // The same for a density at R^3 voxels: a voxel for every 32 rows, and enough work for

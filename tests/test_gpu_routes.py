@@ -289,3 +289,67 @@ def test_calls_under_capture():
         assert torch.equal(a, b)
     for a, b in zip(close, ref_close):
         _close(a, b)
+
+
+def _fine_coarse(L, n, pixels):
+    """A bounded scene whose coarse grid is about as fine as the steps, with n rays."""
+    from paper_2407_10482_gb300 import ngprt as ng
+    cfg = S.small_config(L=L, N=S.level_resolutions(64, 128, L), T_log2=16, R_C=64, blob_std=(0.05, 0.15), W=160, H=96)
+    sc = S.make_scene(cfg)
+    ds = ng.DeviceScene(cfg, sc.tables, sc.coarse, sc.mlp_w)
+    occ = ng.DeviceOcc(sc.occ, cfg.R_O, cfg.n_occ_levels)
+    if pixels:
+        rays = dict(cams=S.orbit_cameras(cfg, 3, azimuth0=5.0), W=cfg.W, H=cfg.H,
+                    pixel_ids=torch.as_tensor(S.random_pixels(n, 3, cfg.W, cfg.H, 2)).cuda())
+        src = (*ng.cameras_struct(rays["cams"], cfg.W, cfg.H), rays["pixel_ids"], None, None)
+    else:
+        o, d = (torch.as_tensor(x).cuda() for x in S.random_rays(n, 3, True))
+        rays, src = dict(rays_o=o, rays_d=d), (None, 0, None, o, d)
+    return ng, ds, occ, S.default_options(cfg), rays, src
+
+
+@pytest.mark.parametrize("L,n,pixels", [(2, 20000, False), (2, (1 << 17) + 33, True), (4, 20000, False),
+                                        (4, (1 << 15) + 33, False), (16, 5001, True), (16, (1 << 15) + 33, True)])
+def test_reverse_pass_on_a_fine_coarse_grid(L, n, pixels):
+    """On both sides of the sizes from which records serve a coarse grid as fine as the
+    steps."""
+    ng, ds, occ, opts, rays, src = _fine_coarse(L, n, pixels)
+    ro, rend = ng.render_opts(opts), ng.Renderer(ds, occ)
+    out = rend.render(opts, state=True, **rays)
+    gen = torch.Generator(device="cuda")
+    gen.manual_seed(1)
+    d_rgb = torch.randn(n, 3, device="cuda", generator=gen)
+    got = []
+    for need in (ng.ngprt_render_backward_scratch_bytes(ds.struct, ro, n),
+                 ng.ngprt_render_backward_workspace_bytes(ds.struct, ro, n)):
+        g = [torch.zeros_like(t) for t in (ds.tables, ds.coarse, ds.mlp_w)]
+        ws = torch.empty(need, dtype=torch.uint8, device="cuda")
+        ng.ngprt_render_backward(ds.struct, occ.struct, *src, n, ro, out["state"], d_rgb, None, None, *g, ws)
+        got.append(g)
+    for a, b in zip(*got):
+        _close(a, b)
+
+
+@pytest.mark.parametrize("pixels", [True, False])
+def test_marks_of_two_large_levels(pixels):
+    """2 levels of 2^20 rows: pixel lists take the density plane, free rays do not."""
+    from paper_2407_10482_gb300 import ngprt as ng
+    cfg = S.hd_config(L=2, N=[128, 1024], T_log2=19, R_O=64, n_occ_levels=4, W=320, H=200)
+    sc = S.make_scene(cfg)
+    ds = ng.DeviceScene(cfg, sc.tables, sc.coarse, sc.mlp_w)
+    docc = ng.DeviceOcc(sc.occ, cfg.R_O, cfg.n_occ_levels)
+    ro, n = ng.render_opts(S.default_options(cfg)), 40000
+    assert ng.ngprt_density_scratch_bytes(ds.struct, n) > 0
+    if pixels:
+        src = (*ng.cameras_struct(S.orbit_cameras(cfg, 2, azimuth0=5.0), cfg.W, cfg.H),
+               torch.as_tensor(S.random_pixels(n, 2, cfg.W, cfg.H, 2)).cuda(), None, None)
+    else:
+        o, d = (torch.as_tensor(x).cuda() for x in S.random_rays(n, 3, False))
+        src = (None, 0, None, o, d)
+    v = [torch.zeros(64 ** 3, dtype=torch.uint8, device="cuda") for _ in range(2)]
+    ng.ngprt_occupancy_visibility(ds.struct, docc.struct, *src, n, ro, 1e-3, 64, v[0])
+    st = C.c_void_p(torch.cuda.current_stream().cuda_stream)
+    assert ng.lib().ngprt_occupancy_visibility(
+        C.byref(ds.struct), C.byref(docc.struct), src[0], src[1], _ptr(src[2]), _ptr(src[3]), _ptr(src[4]), n,
+        C.byref(ro), C.c_float(1e-3), 64, _ptr(v[1]), st) == 0
+    assert torch.equal(v[0], v[1]) and int(v[0].sum()) > 0
