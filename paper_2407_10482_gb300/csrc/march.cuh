@@ -1267,9 +1267,9 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
         //    4096 FP32 rays of 13 samples: 32 lanes 143, 16 85, one 230; of 20 samples 326
         //    and 325; FP16 98, 47 and 195).
         //  - 16 levels, 4 and 8 lanes 2.4 (hd, image of 14400: 8 lanes 575, 4 631, one 1850).
-        //  - 16 levels, 2 lanes 2.4 for images, 2.0 for lists, whose neighbours share less
-        //    (57 k pixels of an image 1387 against 1787; random ones 65 k 2334 against 1889);
-        //    FP16 tables never (57 k: 1203 against 983).
+        //  - 16 levels, 2 lanes 2.4, and 2.0 for pixel lists (57 k pixels of an image 1387
+        //    against 1787, 90 k free BF16 rays 1597 against 1840; random pixels, 65 k 2334
+        //    against 1889); FP16 tables never (57 k: 1203 against 983).
         //  - up to 8 levels the chains are shorter: never 2 lanes (8 levels, 68 k BF16 rays
         //    731 against 508); 8 lanes 1.6, 4 lanes 1.8 for FP32 and 1.2 for 16-bit tables (8
         //    levels: 20 k free FP32 rays 358 at 4 lanes, 624 at one; FP16, 25 k pixels 573
@@ -1287,7 +1287,7 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
         if (!room_cache[dev]) room_cache[dev] = resident_blocks(march_group_kernel<L, DT, AGG>, shm);
         const int64_t room = (int64_t)room_cache[dev] * 128;
         const auto most = [&](int g) {
-            if (!kShort) return g == 1 ? (DT == NGPRT_F16 ? 0 : p.mode == 0 ? 24 : 20) : g < 4 ? 24 : 12;
+            if (!kShort) return g == 1 ? (DT == NGPRT_F16 ? 0 : p.mode != 1 ? 24 : 20) : g < 4 ? 24 : 12;
             if (g == 1) return 0;
             if (p.g.bounded) return 18;
             if (g > 3) return 12;
@@ -1309,14 +1309,20 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
         // 1487 and 1495, 1932 and 1866).  Lists take them where they need no turn more than
         // kBlocks blocks would: a warp of unrelated rays is as long as its longest, so that
         // every turn is whole (random pixels, FP16, 16 levels: 100 k 1992 us in two turns of 5
-        // blocks, 1499 in one of 8; FP32, 140 k, two turns either way: 3742 and 4224).
+        // blocks, 1499 in one of 8; FP32, 140 k, two turns either way: 3742 and 4224).  Free
+        // rays on FP32 stacks of more than 8 levels take them always: with nothing shared, the
+        // coarse rows that a group of gates reads again miss L1 (2^18 rays, 80 M rows: 11.8 ms
+        // at 7 blocks, 10.4 at 5; hd 7.02 and 6.99).
         constexpr size_t wshm =
             (size_t)gate_floats<L, DT, AGG, march_gates<L, DT, kWideBlocks>()>() * 128 * sizeof(float);
         static int wide_cache[16] = {0}, full_cache[16] = {0};
         if (!wide_cache[dev]) wide_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kWideBlocks>, wshm);
         if (!full_cache[dev]) full_cache[dev] = resident_blocks(march_kernel<L, DT, AGG, kBlocks>, shm);
         const int64_t wide = (int64_t)wide_cache[dev] * 128, full = (int64_t)full_cache[dev] * 128;
-        const bool few = p.mode == 0 ? rays * 2 <= wide * 3 : rays <= wide || (rays > full && rays <= 2 * wide);
+        const bool few = p.mode == 0   ? rays * 2 <= wide * 3
+                         : p.mode == 2 && DT == NGPRT_F32 && L > 8
+                             ? true
+                             : rays <= wide || (rays > full && rays <= 2 * wide);
         if (few && !p.fb_a_hat) {
             if (p.tile_counter && grid.x > (unsigned)wide_cache[dev]) grid.x = (unsigned)wide_cache[dev];
             march_kernel<L, DT, AGG, kWideBlocks><<<grid, 128, wshm, st>>>(p);
