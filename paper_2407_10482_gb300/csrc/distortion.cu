@@ -85,7 +85,8 @@ struct DistBwdSampler {
     int skip;  // samples whose gradients are elsewhere already
     __device__ __forceinline__ bool sample(const float u[3], float t, float delta) {
         float f[8];
-        sample_features<L, NGPRT_F32>(g, u, attn_mode, f, gates, blockDim.x);
+        sample_features<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V, false, false, kGatesUpFront>(g, u, attn_mode, f, gates,
+                                                                                         blockDim.x);
         const float sigma = expf(f[0]);
         const float trans = expf(-sigma * delta);
         const float w = T * (1.0f - trans);
@@ -137,8 +138,7 @@ __global__ void __launch_bounds__(128, !kList && L == 8 ? 5 : 0) distortion_back
 // set), or NULL.
 template <int L>
 void launch_dist(bool backward, const DistParams& p, dim3 grid, void* records, float* g_plane, cudaStream_t st) {
-    const size_t shm =
-        (size_t)(backward ? gate_floats<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V>() : 2 * L) * 128 * sizeof(float);
+    const size_t shm = (size_t)gate_floats<L, NGPRT_F32, NGPRT_AGG_SEPARATE_V, kGatesUpFront>() * 128 * sizeof(float);
     if (!backward) {
         if (p.m.plane) {
             static int cache[16] = {0};

@@ -58,10 +58,19 @@ __device__ __forceinline__ void distortion_ray(const DistParams& p, const Weight
     }
 }
 
-// Shared gates of 16 levels at 3 blocks per SM (168 registers): left alone the compiler takes
-// 96 and spills (16384 rays 667 us against 568).
+// Blocks per SM where the compiler's own choice of registers is slow (0: its choice).  Shared
+// gates of 16 levels: 3 (168 registers; with its 96 it spills, 16384 rays 667 us against
+// 568).  Eq. 8 of up to 2 levels: 7 (72 registers; 2 levels, paper shape, 4096 free rays 605
+// us, 842 as it comes, 750 at 8 blocks); of 8 levels: 5 (96 registers; 2^18 pixels 2261 us,
+// 2521 as it comes).
 template <int L, int AGG>
-__global__ void __launch_bounds__(128, L == 16 && AGG == NGPRT_AGG_SHARED_V ? 3 : 0)
+constexpr int distortion_blocks() {
+    if (AGG == NGPRT_AGG_SHARED_V) return L == 16 ? 3 : 0;
+    return AGG != NGPRT_AGG_SEPARATE_V ? 0 : L <= 2 ? 7 : L == 8 ? 5 : 0;
+}
+
+template <int L, int AGG>
+__global__ void __launch_bounds__(128, distortion_blocks<L, AGG>())
     distortion_kernel(const __grid_constant__ DistParams p) {
     extern __shared__ float gate_smem[];
     using Weights = ForwardSampler<L, NGPRT_F32, AGG, kGatesUpFront>;

@@ -185,7 +185,8 @@ constexpr int gate_group() {
 // The group of the other passes that interpolate all channels (regulariser, visibility marks,
 // density grid, proposal targets): all gates up front.  They run one ray or voxel a lane
 // through the general march, where the loads of a group come on top of every level's chain
-// (hd, us up front and by groups: regulariser of 16384 random pixels 1207 and 2221, marks
+// (hd, us up front and by groups: regulariser of 16384 random pixels 1207 and 2221, its
+// one-kernel reverse pass of 2^18 28580 and 29470, marks
 // BF16 802 and 1216, density at 32^3 FP32 32 and 39, FP16 19 and 27).
 constexpr int kGatesUpFront = 0;
 // Blocks per SM of those marches: FP32 stacks of more than 8 levels need the registers of 5
