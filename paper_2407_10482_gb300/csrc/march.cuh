@@ -168,14 +168,15 @@ constexpr int kScatterUnroll = NGPRT_SCATTER_UNROLL;
 // gathers live on.  hd scene: BF16 tables (1283 x 721) 4.69 ms with groups of 4, 4.76 with
 // 2, 4.99 one by one, 7.24 with all logits up front (460 bytes of spills); FP16 1080p 6.56,
 // 6.81, 7.38 and 6.66; FP32 1080p 11.57, 11.63, 11.41 and 12.5, and one by one it is.
-// Stacks of 1, 2 or 3 levels keep all logits up front, with the gates in shared memory: there
-// are few of them, and their rows are too narrow for wide loads of a group (paper shape,
-// L = 2: FP16 3.25 ms against 3.47, FP32 4.71 against 5.12; BF16 3.74 against 9.73, where
-// the warp's lanes no longer sampled together).  So do FP32 tables of up to 8 levels (1283 x
-// 721: L = 4 617 us against 706, L = 8 3.03 ms against 3.15).
+// Stacks of up to 4 levels keep all logits up front, with the gates in shared memory: there
+// are few of them, and the rows of 1 to 3 levels are too narrow for wide loads of a group
+// (paper shape, L = 4: FP16 5.87 ms against 6.30, BF16 6.57 against 7.32, 2^18 free FP16 rays
+// 3.56 against 4.46; L = 2: FP16 3.25 against 3.47, FP32 4.71 against 5.12, BF16 3.74 against
+// 9.73, where the warp's lanes no longer sampled together).  So do FP32 tables of up to 8
+// levels (1283 x 721: L = 4 617 us against 706, L = 8 3.03 ms against 3.15).
 template <int L, int DT, int AGG>
 constexpr bool fly_gates() {
-    if (AGG != NGPRT_AGG_SEPARATE_V || L < 4) return false;
+    if (AGG != NGPRT_AGG_SEPARATE_V || L <= 4) return false;
     return DT == NGPRT_F32 ? L > 8 : DT == NGPRT_BF16 || L % 4 == 0;
 }
 template <int L, int DT>
