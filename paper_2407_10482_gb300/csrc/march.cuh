@@ -1265,9 +1265,9 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
         // which pays even where the blocks take a second turn, and stops to when the GPU is
         // full of rays anyway.  In tenths of the threads that are resident at once, up to
         // how many 2^g lanes are taken (us; "one" is a ray per lane):
-        //  - 16 and 32 lanes 1.2: samples past a ray's end cost as much as the others (hd,
-        //    4096 FP32 rays of 13 samples: 32 lanes 143, 16 85, one 230; of 20 samples 326
-        //    and 325; FP16 98, 47 and 195).
+        //  - 32 lanes 1.2: samples past a ray's end cost as much as the others (hd, 4096 FP32
+        //    rays of 13 samples: 32 lanes 143, 16 85, one 230; of 20 samples 326 and 325; FP16
+        //    98, 47 and 195).  16 lanes 1.8.
         //  - 16 levels, 4 and 8 lanes 2.4 (hd, image of 14400: 8 lanes 575, 4 631, one 1850).
         //  - 16 levels, 2 lanes 2.4, and 2.0 for pixel lists (57 k pixels of an image 1387
         //    against 1787, 90 k free BF16 rays 1597 against 1840; random pixels, 65 k 2334
@@ -1289,10 +1289,10 @@ void launch_march_dt(const MarchParams& p, dim3 grid, cudaStream_t st) {
         if (!room_cache[dev]) room_cache[dev] = resident_blocks(march_group_kernel<L, DT, AGG>, shm);
         const int64_t room = (int64_t)room_cache[dev] * 128;
         const auto most = [&](int g) {
-            if (!kShort) return g == 1 ? (DT == NGPRT_F16 ? 0 : p.mode != 1 ? 24 : 20) : g < 4 ? 24 : 12;
+            if (!kShort) return g == 1 ? (DT == NGPRT_F16 ? 0 : p.mode != 1 ? 24 : 20) : g < 4 ? 24 : g == 4 ? 18 : 12;
             if (g == 1) return 0;
             if (p.g.bounded) return 18;
-            if (g > 3) return 12;
+            if (g > 3) return g == 4 ? 18 : 12;
             if (L == 1 && DT != NGPRT_F32) return 18;
             return g == 3 ? 16 : L <= 4 ? 0 : DT == NGPRT_F32 ? 18 : 12;
         };
